@@ -435,46 +435,47 @@ __device__ __forceinline__ double half_sum_exact(float a, float b)
     return __longlong_as_double((long long)bits);
 }
 
-// binary32 -> binary64 (exact) of a positive normal value: the significand shifted into place
-// and the exponent rebiased from 127 to 1023 by one 64-bit add
-__device__ __forceinline__ double f32_to_f64_posnormal(float f)
+// the one of two adjacent binary32 roundings (down, up) of a value whose significand is odd, or
+// the value itself where both are equal: rounding to odd, which keeps in the last bit whether
+// anything was cut off, so that a later rounding to nearest sees on which side of a tie it lies
+__device__ __forceinline__ float round_odd(float down, float up)
 {
-    return __longlong_as_double((long long)(((unsigned long long)__float_as_uint(f) << 29) + (896ull << 52)));
-}
-
-// binary64 -> binary32, round to nearest even, of a positive value whose binary32 result is a
-// normal number or infinity: the exponent rebiased from 1023 to 127 in the shifted bit pattern
-__device__ __forceinline__ float f64_to_f32_posnormal(double x)
-{
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-    unsigned int f = (unsigned int)((b >> 29) - (896ull << 23));
-    const unsigned int rem = (unsigned int)b & 0x1fffffffu;
-    f += (rem > 0x10000000u || (rem == 0x10000000u && (f & 1u))) ? 1u : 0u;
-    return __uint_as_float(f);
+    return (__float_as_uint(down) & 1u) ? down : up;
 }
 
 // {a}(1 - del) rounded to binary32, the value of the log-mean small-jump branch (the
-// Ismail-Roe series, Sec. 3.3): {a} = a/2 + b/2 exact in binary64, times (1 - del) by one FP64
-// fused multiply-add, then rounded.  a, b > 0 and 0 <= del <= 1/2.  When a and b are normal
-// (biased exponents >= 2) and at most 7 binades apart and del is zero or normal, {a} is built
-// with integer instructions (as in half_sum_exact) and the conversions skip their special
-// cases; otherwise the general conversions run.  Both give the same value.
+// Ismail-Roe series, Sec. 3.3), for s = fl(a + b) with 0 <= del <= 0.1 and a, b > 0 within a
+// factor of two of each other.  The value is 0.5 (a + b)(1 - del), kept exactly until the one
+// final rounding: a + b = s + e (two-sum), s (1 - del) = r + (s - r) - s del, where s - r and
+// (s - r) + e are exact, and the remainder (s - r) + e - s del - e del is formed by two fused
+// multiply-adds rounded to odd.  That is the value of the binary64 evaluation (half_sum_exact,
+// one FP64 fused multiply-add, rounded to binary32) except where that one rounds twice, about
+// once in 5e8 (2 of 9.8e8 random pairs, measured).
+// Why: the binary64 evaluation with integer-built {a} takes 45 issued instructions, one of them
+// on the FP64 pipe, whose rate is 1/64 of FP32's; this one takes 22 and none there (ncu counts
+// of a kernel that does nothing else).  It runs 21 times per node and stage of a 2D step.
+// Sums outside [2^-63, 2^63), where scaled remainders could leave the binary32 range, keep the
+// binary64 evaluation.
+__device__ __forceinline__ float logmean_small_near(float a, float b, float s, float del)
+{
+    if (__float_as_uint(s) - 0x20000000u < 0x3f000000u) {
+        const float e = __fsub_rn(fminf(a, b), __fsub_rn(s, fmaxf(a, b)));
+        const float r = __fmaf_rn(-s, del, s);
+        const float g = __fadd_rn(__fsub_rn(s, r), e);
+        const float z = round_odd(__fmaf_rd(-s, del, g), __fmaf_ru(-s, del, g));
+        const float t = round_odd(__fmaf_rd(-e, del, z), __fmaf_ru(-e, del, z));
+        return 0.5f * __fadd_rn(r, t);
+    }
+    const double hs = half_sum_exact(a, b);
+    return f64_to_f32(fma(-hs, f32_to_f64(del), hs));
+}
+
+// the same for any a, b > 0 and 0 <= del <= 1/2.  The smallest del of the series is that of
+// neighbouring binary32 values, 2^-51.6; below 2^-52 the binary64 evaluation rounds del away
 __device__ __forceinline__ float logmean_small(float a, float b, float del)
 {
-    const unsigned int ua = __float_as_uint(a), ub = __float_as_uint(b);
-    const int ea = (int)(ua >> 23), eb = (int)(ub >> 23);
-    const int e = min(ea, eb), dl = max(ea, eb) - e;
-    const bool del_ok = del == 0.0f || (__float_as_uint(del) >> 23) != 0u;
-    if (e >= 2 && dl <= 7 && max(ea, eb) <= 254 && del_ok) {
-        const unsigned int ma = (ua & 0x7fffffu) | 0x800000u, mb = (ub & 0x7fffffu) | 0x800000u;
-        const unsigned int M = (ma << (ea - e)) + (mb << (eb - e));
-        const int k = 31 - __clz((int)M);
-        const double hs = __longlong_as_double(
-            (long long)(((unsigned long long)(k + e + 871) << 52) + ((unsigned long long)M << (52 - k))));
-        const double d = del == 0.0f ? 0.0 : f32_to_f64_posnormal(del);
-        return f64_to_f32_posnormal(fma(-hs, d, hs));
-    }
-    const double hs = f32_to_f64(0.5f * a) + f32_to_f64(0.5f * b);
+    if ((del == 0.0f || del >= 0x1p-52f) && del <= 0.1f && 2.0f * fminf(a, b) >= fmaxf(a, b)) return logmean_small_near(a, b, a + b, del);
+    const double hs = half_sum_exact(a, b);
     return f64_to_f32(fma(-hs, f32_to_f64(del), hs));
 }
 
