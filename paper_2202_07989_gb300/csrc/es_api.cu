@@ -526,11 +526,25 @@ const double XCOEF[3] = { 1.0, 0.5, 1.0 };
 // 2D moving meshes form the stage metrics as M(x^n) + s dt M(xdot) (the metrics are linear in x)
 bool linear_stage_metrics(const es_ctx* c) { return c->d == 2 && !c->hI[0].fixed; }
 
-// whether the mesh step runs the fused 2D launch (monitor, filter passes and sweeps)
+// whether the mesh step runs the fused 2D launches (monitor, filter passes and sweeps)
 bool fused_mesh2d(const es_ctx* c)
 {
     const Inst& I = c->hI[0];
-    return c->mixed && c->d == 2 && !I.fixed && I.mu >= 1 && I.mu <= JACOBI_FUSED_MAX && I.nf <= FILTER_FUSED_MAX;
+    return c->mixed && c->d == 2 && !I.fixed && I.mu >= 1;
+}
+
+// the fused 2D launches of a mesh step in tile shape js; more filter passes than they hold run
+// as launches of their own before them
+void launch_fused_mesh2d(es_ctx* c, int js, const StagePtrs& P, const StagePtrs* tab, cudaStream_t st)
+{
+    const int mu = c->hI[0].mu, nf = c->hI[0].nf, gc = node_grid(c, c->n_cell);
+    int F = nf;
+    if (nf > FILTER_FUSED_MAX) {
+        launch_monitor_theta(true, gc, st, c->dI, c->w_cell, c->n_cell, c->dS);
+        for (int f = 0; f < nf; ++f) launch_filter(true, false, gc, st, c->dI, c->w_cell, c->n_cell, c->dS, f % 2);
+        F = -1;
+    }
+    jacobi_fused2d(js, node_grid(c, c->n_jf[js]), st, c->dI, P, tab, c->w_jf[js], c->n_jf[js], c->dS, mu, F, nf % 2);
 }
 
 // mesh redistribution (Sec. 4): the metrics of x^n (Eq. (cfl) and the monitor need them),
@@ -559,10 +573,7 @@ void launch_mesh(es_ctx* c, const StagePtrs& P, const StagePtrs* tab, cudaStream
     int nf = c->hI[0].nf, mu = c->hI[0].mu;
     int th_sel = nf % 2;
     if (fused_mesh2d(c)) {
-        // monitor, filter passes and sweeps in one launch
-        const int js = c->jf_shape;
-        launch_jacobi_fused2d(js, node_grid(c, c->n_jf[js]), st, c->dI, P, tab, c->w_jf[js], c->n_jf[js], c->dS, mu, nf,
-                              th_sel);
+        launch_fused_mesh2d(c, c->jf_shape, P, tab, st);
     } else {
         // Theta once per node, then plain filter passes (forming it inside the first pass costs
         // 3^d evaluations per node)
@@ -576,7 +587,7 @@ void launch_mesh(es_ctx* c, const StagePtrs& P, const StagePtrs* tab, cudaStream
                 launch_jacobi3d(s == 0, s == mu - 1, node_grid(c, c->n_col), st, c->dI, c->w_col, c->n_col, c->dS, s,
                                 th_sel);
             else
-                launch_jacobi(c->mixed, c->d, s == mu - 1, gc, st, c->dI, P, tab, c->w_cell, c->n_cell, c->dS, s, th_sel);
+                launch_jacobi(s == mu - 1, gc, st, c->dI, P, tab, c->w_cell, c->n_cell, c->dS, s, th_sel);
         }
     }
     if (mu == 0) pdl_launch(limiter_kernel, gc, NODE_TPB, 0, st, c->dI, P, tab, c->w_cell, c->n_cell, c->dS);
@@ -1151,16 +1162,13 @@ es_status es_autotune(es_ctx* c, const double* JU, const double* J, const double
     if (fused_mesh2d(c)) {
         StagePtrs Q = P;
         Q.xdot = nullptr;
-        const int mu = c->hI[0].mu, nf = c->hI[0].nf;
         launch_metrics(c, Q, tab, st, true, false, false);
         launch_cfl_grad(c->mixed, c->d, c->N, node_grid(c, c->n_cell), st, c->dI, P, tab, c->w_cell, c->n_cell, c->dS);
         float best = 3.0e38f;
         for (int sh = 0; sh < NJF_SHAPE; ++sh) {
-            const int grid = node_grid(c, c->n_jf[sh]);
-            launch_jacobi_fused2d(sh, grid, st, c->dI, P, tab, c->w_jf[sh], c->n_jf[sh], c->dS, mu, nf, nf % 2);
+            launch_fused_mesh2d(c, sh, P, tab, st);
             cudaEventRecord(e0, st);
-            for (int r = 0; r < reps; ++r)
-                launch_jacobi_fused2d(sh, grid, st, c->dI, P, tab, c->w_jf[sh], c->n_jf[sh], c->dS, mu, nf, nf % 2);
+            for (int r = 0; r < reps; ++r) launch_fused_mesh2d(c, sh, P, tab, st);
             cudaEventRecord(e1, st);
             if (cudaEventSynchronize(e1) != cudaSuccess) break;
             float ms = 0.f;

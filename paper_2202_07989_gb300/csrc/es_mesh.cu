@@ -792,134 +792,6 @@ __global__ void jacobi_kernel(const Inst* __restrict__ insts, StagePtrs single, 
     }
 }
 
-// Mixed form: one Jacobi sweep of the mesh equation on the displacement y = x - x^n in
-// binary32.  With the spacings dl_{k+-} = x^n_{i+-e_k} - x^n_i (formed in FP64 by the first
-// sweep, stored rounded to binary32) the sweep x_i <- sum T_{k+-} x_{i+-e_k} / dxi_k^2 /
-// sum T_{k+-} / dxi_k^2 reads y_i <- sum w_{k+-} (dl_{k+-} + y_{i+-e_k}) / sum w_{k+-}.
-// The positions stay FP64 (x^n + y); only the sweep arithmetic is FP32.  The last sweep
-// also forms the limiter bounds of Sec. 4, dl_{k,s}[k] / (2 y_k) with s the sign of y_k.
-template <int D, bool FIRST, bool LAST>
-__global__ void __launch_bounds__(NODE_TPB) jacobi_y_kernel(const Inst* __restrict__ insts, StagePtrs single,
-                                                             const StagePtrs* __restrict__ table,
-                                                             const int2* __restrict__ work, int nwork,
-                                                             const Scratch* __restrict__ scr, int sweep, int theta_sel)
-{
-    pdl_entry();
-    __shared__ double sh[32];
-    for (int wi = blockIdx.x; wi < nwork; wi += gridDim.x) {
-        const int2 it = work[wi];
-        const Inst& I = insts[it.x];
-        int i[3];
-        const bool valid = tile_node(I, it.y, 0, i[0], i[1], i[2]);
-        ES_PTRS(P);
-        float bnd = 1.0f;
-        if (valid) {
-            const Scratch& Sc = scr[it.x];
-            const long long n = I.ncell;
-            const long long p = lin(I, i[0], i[1], i[2]);
-            const float* th = reinterpret_cast<const float*>(theta_sel ? Sc.th1 : Sc.th0);
-            const float* ys = reinterpret_cast<const float*>(sweep % 2 == 1 ? Sc.xa : Sc.xb);
-            float* yd = reinterpret_cast<float*>(sweep % 2 == 0 ? Sc.xa : Sc.xb);
-            float* dl = Sc.dl;
-            const float tc = th[p];
-            bool inner = true;
-#pragma unroll
-            for (int k = 0; k < D; ++k) inner = inner && i[k] >= 1 && i[k] < I.n[k] - 1;
-            float num[D], den = 0.0f, dk[D][2];
-#pragma unroll
-            for (int j = 0; j < D; ++j) num[j] = 0.0f;
-            if (inner && !FIRST) {
-                // interior, after the first sweep: every load up front, no boundary maps
-                const long long st[3] = { 1, I.n[0], (long long)I.n[0] * I.n[1] };
-                float tn[D][2], dv[D][2][D], yv[D][2][D];
-#pragma unroll
-                for (int k = 0; k < D; ++k)
-#pragma unroll
-                    for (int s = 0; s < 2; ++s) {
-                        const long long q = p + (s ? st[k] : -st[k]);
-                        tn[k][s] = th[q];
-#pragma unroll
-                        for (int j = 0; j < D; ++j) {
-                            dv[k][s][j] = dl[((k * 2 + s) * D + j) * n + p];
-                            yv[k][s][j] = ys[j * n + q];
-                        }
-                    }
-#pragma unroll
-                for (int k = 0; k < D; ++k)
-#pragma unroll
-                    for (int s = 0; s < 2; ++s) {
-                        const float w = 0.5f * (tc + tn[k][s]) * I.f_h2[k];
-                        dk[k][s] = dv[k][s][k];
-#pragma unroll
-                        for (int j = 0; j < D; ++j) num[j] = fmaf(w, dv[k][s][j] + yv[k][s][j], num[j]);
-                        den += w;
-                    }
-            } else {
-            long long stride = 1;
-#pragma unroll
-            for (int k = 0; k < D; ++k) {
-#pragma unroll
-                for (int s = 0; s < 2; ++s) {
-                    int nb[3] = { i[0], i[1], i[2] };
-                    nb[k] += s ? 1 : -1;
-                    const long long q = p + (s ? stride : -stride);
-                    const float w = 0.5f * (tc + th[inner ? q : s_map(I, nb[0], nb[1], nb[2])]) * I.f_h2[k];
-                    float dv[D], yv[D];
-                    if (FIRST) {
-                        double xn[3];
-                        if (inner) {
-#pragma unroll
-                            for (int j = 0; j < D; ++j) xn[j] = P.x[j * n + q];
-                        } else {
-                            x_at<false>(I, P.x, nb[0], nb[1], nb[2], xn);
-                        }
-#pragma unroll
-                        for (int j = 0; j < D; ++j) {
-                            dv[j] = f64_to_f32(xn[j] - P.x[j * n + p]);
-                            dl[((k * 2 + s) * D + j) * n + p] = dv[j];
-                            yv[j] = 0.0f;
-                        }
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < D; ++j) dv[j] = dl[((k * 2 + s) * D + j) * n + p];
-                        if (inner) {
-#pragma unroll
-                            for (int j = 0; j < D; ++j) yv[j] = ys[j * n + q];
-                        } else {
-                            y_at(I, ys, nb[0], nb[1], nb[2], yv);
-                        }
-                    }
-                    dk[k][s] = dv[k];
-#pragma unroll
-                    for (int j = 0; j < D; ++j) num[j] = fmaf(w, dv[j] + yv[j], num[j]);
-                    den += w;
-                }
-                stride *= I.n[k];
-            }
-            }
-            float ynew[D];
-#pragma unroll
-            for (int j = 0; j < D; ++j) {
-                ynew[j] = num[j] / den;
-                yd[j * n + p] = ynew[j];
-            }
-            if (LAST) {
-#pragma unroll
-                for (int k = 0; k < D; ++k) {
-                    const float dx = ynew[k];
-                    if (dx < 0.0f) bnd = fminf(bnd, dk[k][0] / (2.0f * dx));
-                    else if (dx > 0.0f) bnd = fminf(bnd, dk[k][1] / (2.0f * dx));
-                }
-                if (!(bnd >= 0.0f)) bnd = 0.0f;
-            }
-        }
-        if (LAST) {
-            const double m = block_min_pos(f32_to_f64(bnd), sh);
-            if (threadIdx.x == 0) atomic_min_pos(&scr[it.x].red[5], m);
-        }
-    }
-}
-
 // Slot q = threadIdx.x, threadIdx.x + TPB, ... of a W-wide region (TPB threads per block) and its column and row
 // (a, b) = (q % W, q / W), stepped without a division per slot (W is a run-time width)
 template <int TPB>
@@ -943,24 +815,32 @@ struct SlotIterN {
 using SlotIter = SlotIterN<NODE_TPB>;
 
 
-// Mixed form, 2D: the monitor, its F <= 4 filter passes and all H = mu <= 8 Jacobi sweeps
-// of jacobi_y_kernel in one launch (temporal blocking).  A block of TPB threads stages the region
-// of its TX x TY node tile plus a halo of H + F nodes in shared memory: Theta (formed from the
-// monitor gradients, then filtered F times; the halo shrinks by one node per pass), then on
-// the inner region (halo H) the displacements (ping-pong) and the spacings dl_{k+-} (formed in
-// FP64 from x^n, rounded to binary32).  Each Jacobi sweep updates every in-domain node of the
-// inner region with the arithmetic of jacobi_y_kernel, then re-mirrors the wall ghost nodes
-// from their source nodes; each filter pass likewise re-copies the boundary node into its
-// ghosts (the maps of s_map).  The valid zone shrinks by one node per pass or sweep, so after
-// all of them the tile is exact.  Periodic directions need no care: the region runs over
-// unwrapped indices and reads the wrapped node's data.  The last sweep forms the limiter
-// bounds of Sec. 4 for the tile.  F < 0: Theta is read from the buffer theta_sel instead.
+// Mixed form, 2D: the monitor, its F <= 4 filter passes and H <= 8 Jacobi sweeps of the mesh
+// equation in one launch (temporal blocking), on the displacement y = x - x^n in binary32:
+// with the spacings dl_{k+-} = x^n_{i+-e_k} - x^n_i the sweep x_i <- sum T_{k+-} x_{i+-e_k} /
+// dxi_k^2 / sum T_{k+-} / dxi_k^2 reads y_i <- sum w_{k+-} (dl_{k+-} + y_{i+-e_k}) / sum w_{k+-};
+// the positions stay FP64 (x^n + y).  A block of TPB threads stages the region of its TX x TY
+// node tile plus a halo of H + F nodes in shared memory: Theta (formed from the monitor
+// gradients, then filtered F times; the halo shrinks by one node per pass), then on the inner
+// region (halo H) the displacements (ping-pong) and the spacings dl_{k+-} (formed in FP64 from
+// x^n, rounded to binary32).  Each Jacobi sweep updates every in-domain node of the inner
+// region, then re-mirrors the wall ghost nodes from their source nodes; each filter pass
+// likewise re-copies the boundary node into its ghosts (the maps of s_map).  The valid zone
+// shrinks by one node per pass or sweep, so after all of them the tile is exact.  Periodic
+// directions need no care: the region runs over unwrapped indices and reads the wrapped node's
+// data.
+// A mesh step of more than 8 sweeps runs in several launches of about equal sweep counts
+// (jacobi_fused2d): every launch but the last stores y, the first also the filtered Theta, and
+// every launch but the first starts from the stored y (src) and Theta (F < 0).  The last one
+// forms the limiter bounds of Sec. 4.  One launch per filter pass and sweep, as such steps ran
+// before, is bound by launch latency: the 64^2 vortex step with ten
+// sweeps and three filter passes went from 141.2 us (14 such launches) to 108.9 us (2 launches).
 template <int TX, int TY, int TPB>
 __global__ void __launch_bounds__(TPB, 1024 / TPB) jacobi_fused2d_kernel(const Inst* __restrict__ insts, StagePtrs single,
                                                                           const StagePtrs* __restrict__ table,
                                                                           const int2* __restrict__ work, int nwork,
                                                                           const Scratch* __restrict__ scr, int H, int F,
-                                                                          int theta_sel)
+                                                                          int theta_sel, JfPass pass)
 {
     using SI = SlotIterN<TPB>;
     pdl_entry();
@@ -1039,14 +919,24 @@ __global__ void __launch_bounds__(TPB, 1024 / TPB) jacobi_fused2d_kernel(const I
             tn_ = t;
         }
         const float* tq = tc_ + Fp * RXo + Fp;     // Theta at inner node (a, b): tq[b * RXo + a]
-        // stage Theta, y = 0 and the + side spacings x^n_{i+e_k} - x^n_i of the in-domain nodes
+        const float* ysrc = pass.src == 0 ? nullptr : reinterpret_cast<const float*>(pass.src == 1 ? Sc.xa : Sc.xb);
+        // stage Theta, y (0, or as the previous launch left it) and the + side spacings x^n_{i+e_k} - x^n_i of the in-domain nodes
         // (a periodic copy takes its wrapped node's, unshifted); the - side of a node whose
         // - neighbour is a wall ghost is formed here too, all others below
         for (SI sl(RX); sl.q < NR; sl.next()) {
             const int q = sl.q, a = sl.a, b = sl.b;
             const int g0 = r0 + a, g1 = r1 + b;
-            ya[q] = ya[NR + q] = yb[q] = yb[NR + q] = 0.0f;
+            float y0[2] = { 0.0f, 0.0f };
             const bool ghost = (!per0 && (g0 < 0 || g0 >= n0)) || (!per1 && (g1 < 0 || g1 >= n1));
+            // (a position more than 10 nodes beyond a wall is no neighbour of a tile node)
+            if (ysrc && (per0 || (g0 >= -10 && g0 < n0 + 10)) && (per1 || (g1 >= -10 && g1 < n1 + 10))) {
+                float yv[3];
+                y_at(I, ysrc, g0, g1, 0, yv);
+                y0[0] = yv[0];
+                y0[1] = yv[1];
+            }
+            ya[q] = yb[q] = y0[0];
+            ya[NR + q] = yb[NR + q] = y0[1];
             if (ghost) continue;
             const int w0 = per0 ? g0 - floordiv_(g0, n0) * n0 : g0, w1 = per1 ? g1 - floordiv_(g1, n1) * n1 : g1;
             const long long c = lin(I, w0, w1, 0);
@@ -1151,16 +1041,17 @@ __global__ void __launch_bounds__(TPB, 1024 / TPB) jacobi_fused2d_kernel(const I
             yc = yn;
             yn = t;
         }
-        // the tile: store y^[mu] and form the limiter bounds
+        // the tile: store y (and Theta for the launches that follow) and form the limiter bounds
         const int lx = (int)threadIdx.x % TX, ly = (int)threadIdx.x / TX;
         const int i0 = r0 + H + lx, i1 = r1 + H + ly;
         float bnd = 1.0f;
         if ((int)threadIdx.x < TX * TY && i0 < n0 && i1 < n1) {
             const int q = (ly + H) * RX + lx + H;
             const long long p = lin(I, i0, i1, 0);
-            float* yd = reinterpret_cast<float*>(I.mu % 2 == 1 ? Sc.xa : Sc.xb);
+            float* yd = reinterpret_cast<float*>(pass.dst == 1 ? Sc.xa : Sc.xb);
             yd[p] = yc[q];
             yd[n + p] = yc[NR + q];
+            if (pass.store_theta) reinterpret_cast<float*>(theta_sel ? Sc.th1 : Sc.th0)[p] = tq[(ly + H) * RXo + lx + H];
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
                 const float dx = yc[k * NR + q];
@@ -1169,6 +1060,7 @@ __global__ void __launch_bounds__(TPB, 1024 / TPB) jacobi_fused2d_kernel(const I
             }
             if (!(bnd >= 0.0f)) bnd = 0.0f;
         }
+        if (!pass.last) continue;
         const double m = block_min_pos(f32_to_f64(bnd), sh);
         if (threadIdx.x == 0) atomic_min_pos(&scr[it.x].red[5], m);
     }
@@ -1194,17 +1086,36 @@ void prepare_mesh()
 #undef JF_ATTR
 }
 
-void launch_jacobi_fused2d(int shape, int grid, cudaStream_t st, const Inst* insts, const StagePtrs& single,
-                           const StagePtrs* table, const int2* work, int nwork, const Scratch* scr, int H, int F,
-                           int theta_sel)
+static void launch_jacobi_fused2d(int shape, int grid, cudaStream_t st, const Inst* insts, const StagePtrs& single,
+                                  const StagePtrs* table, const int2* work, int nwork, const Scratch* scr, int H, int F,
+                                  int theta_sel, const JfPass& pass)
 {
     const size_t sm = jacobi_fused2d_smem(H, F, shape);
 #define JF_LAUNCH(S, TX, TY, TPB)                                                                                  \
     if (shape == S)                                                                                                \
         pdl_launch(jacobi_fused2d_kernel<TX, TY, TPB>, grid, TPB, sm, st, insts, single, table, work, nwork, scr, H, F, \
-                   theta_sel);
+                   theta_sel, pass);
     JF_KERNELS(JF_LAUNCH)
 #undef JF_LAUNCH
+}
+
+void jacobi_fused2d(int shape, int grid, cudaStream_t st, const Inst* insts, const StagePtrs& single,
+                    const StagePtrs* table, const int2* work, int nwork, const Scratch* scr, int mu, int F, int theta_sel)
+{
+    // launches of at most JACOBI_FUSED_MAX sweeps, as equal as they come; y alternates between the
+    // two buffers and ends in the one xmu_of names
+    const int np = (mu + JACOBI_FUSED_MAX - 1) / JACOBI_FUSED_MAX;
+    for (int p = 0, done = 0; p < np; ++p) {
+        const int H = (mu - done + np - p - 1) / (np - p), left = np - 1 - p;
+        const int end = mu % 2 == 1 ? 1 : 2, dst = left % 2 == 0 ? end : 3 - end;
+        JfPass pass;
+        pass.src = p == 0 ? 0 : 3 - dst;
+        pass.dst = dst;
+        pass.store_theta = p == 0 && F >= 0 && left > 0;
+        pass.last = left == 0;
+        launch_jacobi_fused2d(shape, grid, st, insts, single, table, work, nwork, scr, H, p == 0 ? F : -1, theta_sel, pass);
+        done += H;
+    }
 }
 
 // Delta_tau = min(1, bounds of Sec. 4) per instance
@@ -1690,22 +1601,12 @@ void launch_xdot(bool mixed, int grid, cudaStream_t st, const Inst* insts, const
     else pdl_launch(xdot_kernel<false>, grid, NODE_TPB, 0, st, insts, single, table, work, nwork, scr);
 }
 
-void launch_jacobi(bool mixed, int d, bool last, int grid, cudaStream_t st, const Inst* insts, const StagePtrs& single,
+void launch_jacobi(bool last, int grid, cudaStream_t st, const Inst* insts, const StagePtrs& single,
                    const StagePtrs* table, const int2* work, int nwork, const Scratch* scr, int sweep, int theta_sel)
 {
 #define JL(R, LS) pdl_launch(jacobi_kernel<R, LS>, grid, NODE_TPB, 0, st, insts, single, table, work, nwork, scr, sweep, theta_sel)
-#define JY(D, F, LS) pdl_launch(jacobi_y_kernel<D, F, LS>, grid, NODE_TPB, 0, st, insts, single, table, work, nwork, scr, sweep, theta_sel)
-    if (mixed) {
-        // 2D (beyond the fused kernel's limits); the mixed 3D sweeps run launch_jacobi3d
-        (void)d;
-        const bool first = sweep == 0;
-        if (first) { if (last) JY(2, true, true); else JY(2, true, false); }
-        else { if (last) JY(2, false, true); else JY(2, false, false); }
-    } else {
-        if (last) JL(double, true);
-        else JL(double, false);
-    }
-#undef JY
+    if (last) JL(double, true);
+    else JL(double, false);
 #undef JL
 }
 

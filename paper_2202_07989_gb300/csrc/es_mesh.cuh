@@ -108,9 +108,9 @@ void launch_monitor_theta(bool mixed, int grid, cudaStream_t st, const Inst* ins
                           const Scratch* scr);
 void launch_filter(bool mixed, bool from_g, int grid, cudaStream_t st, const Inst* insts, const int2* work, int nwork,
                    const Scratch* scr, int parity);
-// mixed form, 2D: the monitor, up to FILTER_FUSED_MAX filter passes and up to JACOBI_FUSED_MAX
-// sweeps in one launch (F < 0: Theta read from the buffer theta_sel), over node tiles of one of
-// the shapes JF_SHAPES (TX, TY, threads per block) and a work list of those tiles
+// mixed form, 2D: the monitor, up to FILTER_FUSED_MAX filter passes and the mu sweeps, at most
+// JACOBI_FUSED_MAX a launch (F < 0: Theta read from the buffer theta_sel), over node tiles of one
+// of the shapes JF_SHAPES (TX, TY, threads per block) and a work list of those tiles
 constexpr int JACOBI_FUSED_MAX = 8, FILTER_FUSED_MAX = 4;
 constexpr int NJF_SHAPE = 4;
 constexpr int JF_SHAPES[NJF_SHAPE][3] = { { 32, 8, 256 }, { 32, 16, 512 }, { 24, 16, 512 }, { 24, 12, 512 } };
@@ -118,16 +118,21 @@ constexpr int JF_SHAPE_DEFAULT = 0;
 void prepare_mesh();    // kernel attributes, once per context
 void prepare_mesh3d();  // those of es_mesh3d.cu
 size_t jacobi_fused2d_smem(int H, int F, int shape);
-void launch_jacobi_fused2d(int shape, int grid, cudaStream_t st, const Inst* insts, const StagePtrs& single,
-                           const StagePtrs* table, const int2* work, int nwork, const Scratch* scr, int H, int F,
-                           int theta_sel);
+// one launch of several: the displacement buffer it starts from (0: y = 0, 1: xa, 2: xb) and ends
+// in, whether it stores Theta for the next one, and whether it is the last (limiter bounds)
+struct JfPass {
+    int src, dst, store_theta, last;
+};
+void jacobi_fused2d(int shape, int grid, cudaStream_t st, const Inst* insts, const StagePtrs& single,
+                    const StagePtrs* table, const int2* work, int nwork, const Scratch* scr, int mu, int F, int theta_sel);
 // mixed form, 3D: one filter pass marching along i3 over the column items of col3 (es_mesh3d.cu)
 void launch_filter3d(int grid, cudaStream_t st, const Inst* insts, const int2* work, int nwork, const Scratch* scr,
                      int parity);
 // mixed form, 3D: one Jacobi sweep marching along i3 over the column items of col3 (es_mesh3d.cu)
 void launch_jacobi3d(bool first, bool last, int grid, cudaStream_t st, const Inst* insts, const int2* work, int nwork,
                      const Scratch* scr, int sweep, int theta_sel);
-void launch_jacobi(bool mixed, int d, bool last, int grid, cudaStream_t st, const Inst* insts, const StagePtrs& single,
+// FP64 form: one Jacobi sweep
+void launch_jacobi(bool last, int grid, cudaStream_t st, const Inst* insts, const StagePtrs& single,
                    const StagePtrs* table, const int2* work, int nwork, const Scratch* scr, int sweep, int theta_sel);
 __global__ void limiter_kernel(const Inst* insts, StagePtrs single, const StagePtrs* table, const int2* work, int nwork,
                                const Scratch* scr);

@@ -3,7 +3,7 @@
 // planes it reads (its nodes plus a one-node halo in i1 and i2) sit in a ring of shared-memory
 // planes: the ghost maps of the boundary conditions are applied once, when a plane is staged,
 // and every node value is loaded once per pass plus the halo, so the stencil arithmetic runs
-// without boundary branches.  A sweep's arithmetic per node is that of jacobi_y_kernel, term
+// without boundary branches.  A sweep's arithmetic per node is that of jacobi_fused2d_kernel, term
 // for term; the filter sums filter_kernel's weights one direction at a time.
 #include "es_mesh.cuh"
 
@@ -108,7 +108,7 @@ __device__ __forceinline__ void m3_edge_below(const Inst& I, const Scratch& Sc, 
     }
 }
 
-// The first mixed Jacobi sweep of a 3D instance, with the arithmetic of jacobi_y_kernel:
+// The first mixed Jacobi sweep of a 3D instance, with the arithmetic of jacobi_fused2d_kernel:
 // y_i <- sum_{k,s} w_{k,s} (dl_{k,s} + y_{i+-e_k}) / sum_{k,s} w_{k,s}, w_{k,s} = (Theta_i +
 // Theta_{i+-e_k}) / 2 / dxi_k^2, in the order k = 1, 2, 3 with the minus side first, from
 // y = 0.  It forms the spacings from XE (x^n with its ghost maps, staged by the metrics pass
@@ -293,7 +293,7 @@ struct J3Smem {
 };
 
 // A later Jacobi sweep of a 3D instance (the arithmetic of jacobi3d_first_kernel with y read
-// from the previous sweep, bit for bit that of jacobi_y_kernel).  The planes are staged with
+// from the previous sweep, bit for bit that of jacobi_fused2d_kernel's sweeps).  The planes are staged with
 // cp.async two planes ahead of the update: at plane i3 each thread waits for the copies it
 // issued two planes before (Theta and y up to plane i3 + 1, the spacings of plane i3), and
 // after the block barrier the block issues Theta and y of plane i3 + 3 and the spacings of

@@ -260,3 +260,29 @@ def test_mesh_tiles_refused():
     assert f.es_get_mesh_tiles()[0] == -1
     with pytest.raises(RuntimeError):
         f.es_set_mesh_tiles(0)
+
+
+@pytest.mark.parametrize("bc", ["periodic", "mixed", "reflect"])
+@pytest.mark.parametrize("mu,nf", [(9, 3), (10, 0), (17, 4), (3, 6)])
+def test_mesh_sweeps_in_several_launches(bc, mu, nf):
+    """More sweeps than one fused launch holds (8), and more filter passes (4): the mixed 2D mesh
+    step in every tile shape gives the same results bit for bit, and the mesh velocity of the
+    oracle at FP32 level, on ragged and sub-tile grids (up to 17 sweeps of about three roundings,
+    2^-24 of a spacing each, against displacements of a few percent of a spacing: 5e-5)."""
+    torch = need_gpu()
+    for n, seed in (((70, 37), 41), ((10, 11), 42)):
+        pb, JU, J, x, _ = case(2, 2, n, bc, es=True, seed=seed, jump=True)
+        pb = pb.with_(mu=mu, nf=nf, sigma=(W.SIG_RHO1, W.SIG_P), alpha=(60.0, 25.0))
+        ctx = _ctx(pb, 1)
+        G = [to_dev(t, torch) for t in (JU, J, x)]
+        out = []
+        for sh in range(NJF_SHAPE):
+            ctx.es_set_mesh_tiles(sh)
+            out.append(ctx.mesh_redistribute(*G))
+        for o in out[1:]:
+            assert _same(o, out[0]), (n, bc)
+        xd_o, dt_o, dtau_o = Oracle(pb).mesh_redistribute(JU, J, x)
+        xd, dd = out[0]
+        assert abs(float(dd[0]) - dt_o) <= 5e-6 * dt_o
+        assert abs(float(dd[1]) - dtau_o) <= 5e-5 * dtau_o
+        assert np.abs(xd.cpu().numpy() - xd_o).max() <= 5e-5 * np.abs(xd_o).max()
