@@ -364,46 +364,47 @@ __device__ inline void load_U(const Inst& I, const double* __restrict__ JU, cons
 // at 1/64 of the FP32 rate).  Values below 2^-126 in magnitude become a signed zero;
 // |x| >= 2^128 (after rounding) and infinities become infinities; NaN becomes the
 // canonical binary32 NaN.
+// The fields are moved together: a funnel shift puts the low 8 exponent bits and the top 23
+// significand bits where binary32 has them (the bias differs by 896 = 128 mod 256), and one
+// 64-bit add of just under half a unit, plus the last kept bit, to (result : cut-off bits)
+// rounds to nearest even, its carry stepping the exponent up to infinity.  18 issued
+// instructions where field-by-field assembly took 27 (ncu counts of kernels that do nothing
+// else); a 2D stage converts 22 values per node.
 __device__ __forceinline__ float f64_to_f32(double x)
 {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-    const unsigned int hi = (unsigned int)(b >> 32);
-    const int e = (int)((hi >> 20) & 0x7ffu);
-    const unsigned int sign = hi & 0x80000000u;
-    const unsigned long long mant = b & 0xFFFFFFFFFFFFFull;
-    if (e < 1023 - 126) return __int_as_float((int)sign);
-    if (e > 1023 + 127) return __int_as_float((int)(e == 0x7ff && mant != 0ull ? 0x7fffffffu : (sign | 0x7f800000u)));
-    const unsigned int m = (unsigned int)(mant >> 29);
-    const unsigned int rem = (unsigned int)(mant & 0x1FFFFFFFull);
-    unsigned int f = sign | ((unsigned int)(e - 1023 + 127) << 23) | m;
-    // a carry out of the significand steps the exponent (up to infinity), as rounding must
-    f += (rem > 0x10000000u || (rem == 0x10000000u && (m & 1u))) ? 1u : 0u;
-    return __int_as_float((int)f);
+    const unsigned int hi = (unsigned int)__double2hiint(x), lo = (unsigned int)__double2loint(x);
+    const unsigned int mag = hi & 0x7fffffffu, sign = hi & 0x80000000u;
+    const unsigned int t = __funnelshift_l(lo, hi, 3);
+    unsigned long long w = ((unsigned long long)(((t + 0x40000000u) & 0x7fffffffu) | sign) << 32) | (lo << 3);
+    w += 0x7fffffffu + (t & 1u);
+    unsigned int f = (unsigned int)(w >> 32);
+    if (mag < ((1023u - 126u) << 20)) f = sign;
+    if (mag >= ((1023u + 128u) << 20))
+        f = (mag > 0x7ff00000u || (mag == 0x7ff00000u && lo != 0u)) ? 0x7fffffffu : (sign | 0x7f800000u);
+    return __uint_as_float(f);
 }
 
 // IEEE 754 binary32 -> binary64 (exact), with integer instructions only; subnormals are
-// normalised, infinities kept, NaN keeps its payload with the quiet bit set
+// normalised, infinities kept, NaN keeps its payload with the quiet bit set.  Zeros and normal
+// values take a shift and an exponent offset (16 issued instructions where the branches on the
+// exponent took 31).
 __device__ __forceinline__ double f32_to_f64(float f)
 {
-    const unsigned int b = (unsigned int)__float_as_int(f);
-    const unsigned int e = (b >> 23) & 0xffu;
-    const unsigned int mant = b & 0x7fffffu;
-    const unsigned long long sign = (unsigned long long)(b & 0x80000000u) << 32;
-    unsigned long long d;
-    if (e == 0xffu) {
-        d = sign | 0x7ff0000000000000ull | ((unsigned long long)mant << 29) | (mant ? 0x0008000000000000ull : 0ull);
-    } else if (e == 0u) {
-        if (mant == 0u) {
-            d = sign;
+    const unsigned int b = __float_as_uint(f), mag = b & 0x7fffffffu, sign = b & 0x80000000u;
+    if (mag - 0x800000u >= 0x7f000000u && mag != 0u) {
+        const unsigned int mant = b & 0x7fffffu;
+        unsigned long long d = (unsigned long long)sign << 32;
+        if (mag >= 0x7f800000u) {
+            d |= 0x7ff0000000000000ull | ((unsigned long long)mant << 29) | (mant ? 0x0008000000000000ull : 0ull);
         } else {
             // mant * 2^-149 with its leading one at bit 23 - sh
             const int sh = __clz((int)mant) - 8;
-            d = sign | ((unsigned long long)(897 - sh) << 52) | ((unsigned long long)((mant << sh) & 0x7fffffu) << 29);
+            d |= ((unsigned long long)(897 - sh) << 52) | ((unsigned long long)((mant << sh) & 0x7fffffu) << 29);
         }
-    } else {
-        d = sign | ((unsigned long long)(e + 896u) << 52) | ((unsigned long long)mant << 29);
+        return __longlong_as_double((long long)d);
     }
-    return __longlong_as_double((long long)d);
+    const unsigned int hi = sign | ((mag >> 3) + (mag ? 896u << 20 : 0u));
+    return __hiloint2double((int)hi, (int)(mag << 29));
 }
 
 template <typename R>

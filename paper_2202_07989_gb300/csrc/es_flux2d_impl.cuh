@@ -98,7 +98,7 @@ __device__ __forceinline__ void flux2d_div1(const Inst& I, int i0, int j0, const
         if (i0 + il >= I.n[0] || j0 + jl >= I.n[1]) continue;
         const int fr = jl * (TX + 1) + il + 1;
         double r[NC + 1];
-        node_div<NC, R>(I, fl, NI, gt, fr, fr - 1, I.inv_dxi[0], r);
+        node_div<NC, R>(I, fl, NI, gt, fr, fr - 1, 0, r);
 #pragma unroll
         for (int q = 0; q <= NC; ++q) acc[q * NO + t] = r[q];
     }
@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(FLUX_TPB, (sizeof(R) == 4 ? 3 : 1)) flux2d_ker
             if (i0 + il >= n0 || j0 + jl >= n1) continue;
             const long long id = lin(I, i0 + il, j0 + jl, 0);
             double r[NC + 1];
-            node_div<NC, R>(I, fl, NI, gt, t + TX, t, I.inv_dxi[1], r);
+            node_div<NC, R>(I, fl, NI, gt, t + TX, t, 1, r);
             if (L.mode == MODE_RK) {
 #pragma unroll
                 for (int q = 0; q < NC; ++q)

@@ -644,9 +644,12 @@ __device__ __forceinline__ double rk_stage(const FluxLaunch& L, double q, const 
 // (the J equation), and the p_inf J xi_k/t part of the energy flux added in FP64
 template <int NC, typename R>
 __device__ __forceinline__ void node_div(const Inst& I, const R* fl, int NI, const double* gt, int fr, int fL,
-                                         double inv_dx, double* r)
+                                         int k, double* r)
 {
-    const R rdx = to_r<R>(inv_dx);
+    const double inv_dx = I.inv_dxi[k];
+    R rdx;
+    if constexpr (std::is_same<R, float>::value) rdx = I.f_inv_dxi[k];
+    else rdx = inv_dx;
     r[NC] = -(gt[fr] - gt[fL]) * inv_dx;
 #pragma unroll
     for (int q = 0; q < NC; ++q) r[q] = to_d(-(fl[q * NI + fr] - fl[q * NI + fL]) * rdx);

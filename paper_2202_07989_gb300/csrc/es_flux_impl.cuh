@@ -133,7 +133,6 @@ __global__ void __launch_bounds__(FLUX_TPB, (sizeof(R) == 4 ? (D == 3 ? 4 : 3) :
         const int ts = it.y % ns, ta = (it.y / ns) % nat, tb = it.y / (ns * nat);
         const int s0 = ts * S, a0 = ta * WT;
         const long long ncell = I.ncell;
-        const double inv_dx = I.inv_dxi[k];
         // 2D stage metrics M + s Md with s = mcoef dt (the stage mesh is x^n + s xdot)
         const double sM = (D == 2 && L.mcoef != 0.0) ? L.mcoef * *P.dt : 0.0;
 
@@ -237,7 +236,7 @@ __global__ void __launch_bounds__(FLUX_TPB, (sizeof(R) == 4 ? (D == 3 ? 4 : 3) :
             const long long id = lin(I, idx[0], idx[1], idx[2]);
             const int fr = w * (S + 1) + s + 1, fL = fr - 1;
             double r[NC + 1];
-            node_div<NC, R>(I, fl, NI, gt, fr, fL, inv_dx, r);
+            node_div<NC, R>(I, fl, NI, gt, fr, fL, k, r);
             if (L.mode == MODE_WRITE) {
 #pragma unroll
                 for (int q = 0; q < NC; ++q) P.accU[q * ncell + id] = r[q];
