@@ -815,6 +815,13 @@ struct SlotIterN {
 using SlotIter = SlotIterN<NODE_TPB>;
 
 
+// whether the (unwrapped) node position (g0, g1) is the first or last node of the grid in a direction
+__device__ __forceinline__ bool grid_edge(int g0, int n0, bool per0, int g1, int n1, bool per1)
+{
+    const int w0 = per0 ? g0 - floordiv_(g0, n0) * n0 : g0, w1 = per1 ? g1 - floordiv_(g1, n1) * n1 : g1;
+    return w0 == 0 || w0 == n0 - 1 || w1 == 0 || w1 == n1 - 1;
+}
+
 // Mixed form, 2D: the monitor, its F <= 4 filter passes and H <= 8 Jacobi sweeps of the mesh
 // equation in one launch (temporal blocking), on the displacement y = x - x^n in binary32:
 // with the spacings dl_{k+-} = x^n_{i+-e_k} - x^n_i the sweep x_i <- sum T_{k+-} x_{i+-e_k} /
@@ -892,11 +899,13 @@ __global__ void __launch_bounds__(TPB, 1024 / TPB) jacobi_fused2d_kernel(const I
                 const int g0 = o0 + a, g1 = o1 + b;
                 const bool ghost = (!per0 && (g0 < 0 || g0 >= n0)) || (!per1 && (g1 < 0 || g1 >= n1));
                 if (ghost || a == 0 || a == RXo - 1 || b == 0 || b == RYo - 1) continue;
+                const bool edge = pass.edges && grid_edge(g0, n0, per0, g1, n1, per1);
                 float acc = 0.0f;
 #pragma unroll
                 for (int j2 = -1; j2 <= 1; ++j2) {
                     const int qr = q + j2 * RXo;
-                    const float row = 0.25f * (tc_[qr - 1] + tc_[qr + 1]) + 0.5f * tc_[qr];
+                    float row = 0.25f * (tc_[qr - 1] + tc_[qr + 1]) + 0.5f * tc_[qr];
+                    if (edge) row = __fmaf_rn(0.25f, tc_[qr + 1], __fmaf_rn(0.5f, tc_[qr], 0.25f * tc_[qr - 1]));
                     acc += (j2 == 0 ? 0.5f : 0.25f) * row;
                 }
                 tn_[q] = acc;
@@ -947,8 +956,8 @@ __global__ void __launch_bounds__(TPB, 1024 / TPB) jacobi_fused2d_kernel(const I
                 for (int sd = 0; sd < 2; ++sd) {
                     const int nb0 = w0 + (k == 0 ? (sd ? 1 : -1) : 0), nb1 = w1 + (k == 1 ? (sd ? 1 : -1) : 0);
                     const bool inside = nb0 >= 0 && nb0 < n0 && nb1 >= 0 && nb1 < n1;
-                    const bool wall = !(k == 0 ? per0 : per1) && !inside;
-                    if (sd == 0 && !wall) continue;          // from the neighbour's + side below
+                    const bool wall = !(k == 0 ? per0 : per1) && !inside, seam = pass.edges && !inside;
+                    if (sd == 0 && !wall && !seam) continue;  // from the neighbour's + side below
                     double xn[3];
                     if (inside) {
                         const long long cn = lin(I, nb0, nb1, 0);
@@ -988,6 +997,7 @@ __global__ void __launch_bounds__(TPB, 1024 / TPB) jacobi_fused2d_kernel(const I
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
                 const bool wall = k == 0 ? (!per0 && g0 == 0) : (!per1 && g1 == 0);
+                if (pass.edges && (k == 0 ? g0 - floordiv_(g0, n0) * n0 : g1 - floordiv_(g1, n1) * n1) == 0) continue;
                 if (wall || (k == 0 ? a == 0 : b == 0)) continue;
                 const int qn = q - (k == 0 ? 1 : RX);
 #pragma unroll
@@ -1113,6 +1123,7 @@ void jacobi_fused2d(int shape, int grid, cudaStream_t st, const Inst* insts, con
         pass.dst = dst;
         pass.store_theta = p == 0 && F >= 0 && left > 0;
         pass.last = left == 0;
+        pass.edges = np > 1 || F < 0;
         launch_jacobi_fused2d(shape, grid, st, insts, single, table, work, nwork, scr, H, p == 0 ? F : -1, theta_sel, pass);
         done += H;
     }
