@@ -195,7 +195,10 @@ es_status es_set_tuning(es_ctx* ctx, int k, int shape, int grid);
  * results are bitwise those of the per-direction launches.  es_autotune on a 2D
  * context also times each fused shape and keeps the fused launch when it beats
  * the sum of the best per-direction launches.  A new 2D context starts with the
- * fused launch in shape 0 (16 x 12 tiles, full occupancy).
+ * fused launch in shape 0 (16 x 12 tiles, full occupancy).  On grids of few tiles
+ * a new context, and es_autotune where it measures them faster, run the launch on
+ * smaller tiles (8 x 8, 12 x 8 or 16 x 8) behind the reported shape; a shape set by
+ * es_set_fusion runs as it is.
  * es_get_fusion: fused shape index (-1: per-direction launches), TX, TY, grid
  * (CTAs) and the best fused time per launch the last es_autotune measured (0 if
  * none; set even when the per-direction launches won).  All pointers HOST, one
@@ -209,13 +212,16 @@ es_status es_set_fusion(es_ctx* ctx, int shape, int grid);
 
 /* Tiles of the mixed-form 2D mesh step (the paper has no counterpart; a launch
  * schedule).  The monitor, the filter passes and the Jacobi sweeps of Sec. 4 run
- * in one launch over TX x TY node tiles, each staged in shared memory with a halo
- * of mu + n_f nodes (temporal blocking), in one of 4 shapes: 0: 32 x 8 tiles with
- * 256 threads per block; 1: 32 x 16, 2: 24 x 16, 3: 24 x 12, each with 512.
- * Every node's displacement is formed by the same arithmetic in any tile, so the
- * shape changes no result.  es_autotune on such a context also times every shape
- * on one mesh step of the given state and keeps the fastest.  A new context
- * starts in shape 0.
+ * in one launch (more than 8 sweeps in several) over TX x TY node tiles, each
+ * staged in shared memory with a halo of its sweeps and filter passes (temporal
+ * blocking), in one of 4 shapes: 0: 32 x 8 tiles with 256 threads per block;
+ * 1: 32 x 16, 2: 24 x 16, 3: 24 x 12, each with 512.  Every node's displacement is
+ * formed by the same arithmetic in any tile, so the shape changes no result.
+ * es_autotune on such a context also times every shape on one mesh step of the
+ * given state and keeps the fastest.  A new context reports shape 0 and runs the
+ * tiles that its grid size suggests, smaller ones (16 x 8, 8 x 8) on small grids
+ * among them; es_autotune may keep those behind the reported shape too, and a
+ * shape set by es_set_mesh_tiles runs as it is.
  * es_get_mesh_tiles: shape index, TX, TY, threads per block and the best time per
  * launch the last es_autotune measured (0 if none).  All pointers HOST, one value
  * each; on contexts without the fused mesh step, shape -1 and zeros.

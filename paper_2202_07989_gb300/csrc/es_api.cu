@@ -31,11 +31,12 @@ struct es_ctx {
     int2* w_col = nullptr;  int n_col = 0;     // 3D: column chunks of the kernels marching along i3
     int2* w_flux[3][NSHAPE] = {};          // flux work list per direction and tile shape
     int n_flux[3][NSHAPE] = {};
-    int2* w_fused[NFSHAPE] = {};           // fused 2D stage work list per fused tile shape
-    int n_fused[NFSHAPE] = {};
-    int2* w_jf[NJF_SHAPE] = {};            // mixed 2D: fused mesh-step tiles per shape (JF_SHAPES)
-    int n_jf[NJF_SHAPE] = {};
+    int2* w_fused[NFSHAPE_ALL] = {};           // fused 2D stage work list per fused tile shape
+    int n_fused[NFSHAPE_ALL] = {};
+    int2* w_jf[NJF_SHAPE_ALL] = {};            // mixed 2D: fused mesh-step tiles per shape (JF_SHAPES)
+    int n_jf[NJF_SHAPE_ALL] = {};
     int jf_shape = JF_SHAPE_DEFAULT;
+    int jf_run = -1;                       // the tiles the launch runs on where the library chose others; -1: jf_shape
     float jf_ms = 0.f;
     int* d_first_cell = nullptr;
     double* partial = nullptr;
@@ -63,6 +64,9 @@ struct es_ctx {
     int fused_shape = -1;
     int fused_grid = 0;
     float fused_ms = 0.f;
+    // the tiles a fused launch runs on, where the library chose others (small grids); -1: fused_shape
+    int fused_run = -1;
+    int fused_run_grid = 0;
     std::string err;
     // kernel timing (es_profile)
     bool prof = false;
@@ -307,6 +311,24 @@ long long fused_tiles(const Inst& I, int shape)
     return (long long)((I.n[0] + FSHAPE_TX[shape] - 1) / FSHAPE_TX[shape]) * ((I.n[1] + FSHAPE_TY[shape] - 1) / FSHAPE_TY[shape]);
 }
 
+// The tiles of a context that nobody tuned: shape 0, or the small-grid shape whose waves over the
+// SMs' resident CTAs cost less (FSHAPE_COST).  The arithmetic is the same in every shape.
+void pick_fused(es_ctx* c)
+{
+    c->fused_run = -1;
+    double best = 0.0;
+    for (int sh = 0; sh < NFSHAPE_ALL; ++sh) {
+        if (sh > 0 && sh < NFSHAPE) continue;
+        const int slots = c->sms * flux2d_occ(c, sh);
+        const double cost = (double)((c->n_fused[sh] + slots - 1) / slots) * FSHAPE_COST[sh][c->mixed ? 0 : 1];
+        if (sh == 0 || cost < best) {
+            best = cost;
+            c->fused_run = sh;
+            c->fused_run_grid = slots;
+        }
+    }
+}
+
 // flux tiles of instance I along direction k in tile shape `shape`
 long long flux_tiles(const Inst& I, int k, int shape)
 {
@@ -436,8 +458,9 @@ void launch_residual(es_ctx* c, const StagePtrs& P, const StagePtrs* tab, bool r
         L.insts = c->dI;
         L.single = P;
         L.ptrs = tab;
-        L.work = c->w_fused[c->fused_shape];
-        L.nwork = c->n_fused[c->fused_shape];
+        const int sh = c->fused_run >= 0 ? c->fused_run : c->fused_shape;
+        L.work = c->w_fused[sh];
+        L.nwork = c->n_fused[sh];
         L.k = 0;
         L.mode = rk ? MODE_RK : MODE_WRITE;
         L.a = a;
@@ -446,7 +469,7 @@ void launch_residual(es_ctx* c, const StagePtrs& P, const StagePtrs* tab, bool r
         L.xc = xc;
         L.status = c->status;
         ProfScope ps(c, PC_FLUX2D, st);
-        flux2d_launch(c, L, c->fused_shape, c->fused_grid, st);
+        flux2d_launch(c, L, sh, c->fused_run >= 0 ? c->fused_run_grid : c->fused_grid, st);
         return;
     }
     for (int k = 0; k < c->d; ++k) {
@@ -533,6 +556,22 @@ bool fused_mesh2d(const es_ctx* c)
     return c->mixed && c->d == 2 && !I.fixed && I.mu >= 1;
 }
 
+// The mesh tiles of a context that nobody tuned: least time by the model of JF_COST.  The
+// arithmetic is the same in every shape.
+void pick_mesh_tiles(es_ctx* c)
+{
+    double best = 0.0;
+    for (int sh = 0; sh < NJF_SHAPE_ALL; ++sh) {
+        if (JF_COST[sh] <= 0.0) continue;
+        const int per_sm = (c->n_jf[sh] + c->sms - 1) / c->sms;
+        const double t = JF_COST[sh] * (1.3 * (per_sm / 2) + per_sm % 2);
+        if (c->jf_run < 0 || t < best) {
+            best = t;
+            c->jf_run = sh;
+        }
+    }
+}
+
 // the fused 2D launches of a mesh step in tile shape js; more filter passes than they hold run
 // as launches of their own before them
 void launch_fused_mesh2d(es_ctx* c, int js, const StagePtrs& P, const StagePtrs* tab, cudaStream_t st)
@@ -573,7 +612,7 @@ void launch_mesh(es_ctx* c, const StagePtrs& P, const StagePtrs* tab, cudaStream
     int nf = c->hI[0].nf, mu = c->hI[0].mu;
     int th_sel = nf % 2;
     if (fused_mesh2d(c)) {
-        launch_fused_mesh2d(c, c->jf_shape, P, tab, st);
+        launch_fused_mesh2d(c, c->jf_run >= 0 ? c->jf_run : c->jf_shape, P, tab, st);
     } else {
         // Theta once per node, then plain filter passes (forming it inside the first pass costs
         // 3^d evaluations per node)
@@ -737,18 +776,19 @@ es_status es_create_batch(const es_config* cfgs, int n_inst, es_ctx** out)
             ok = ok && c->w_flux[k][sh];
         }
     if (c->d == 2)
-        for (int sh = 0; sh < NFSHAPE; ++sh) {
+        for (int sh = 0; sh < NFSHAPE_ALL; ++sh) {
             c->w_fused[sh] = build_work(c, [sh](const Inst& I) { return fused_tiles(I, sh); }, c->n_fused[sh]);
             ok = ok && c->w_fused[sh];
         }
     if (c->d == 2 && c->mixed)
-        for (int sh = 0; sh < NJF_SHAPE; ++sh) {
+        for (int sh = 0; sh < NJF_SHAPE_ALL; ++sh) {
             c->w_jf[sh] = build_work(c, [sh](const Inst& I) {
                 return (long long)((I.n[0] + JF_SHAPES[sh][0] - 1) / JF_SHAPES[sh][0]) *
                        ((I.n[1] + JF_SHAPES[sh][1] - 1) / JF_SHAPES[sh][1]);
             }, c->n_jf[sh]);
             ok = ok && c->w_jf[sh];
         }
+    if (c->d == 2 && c->mixed) pick_mesh_tiles(c);
     // per-instance ranges of the cell work list (entropy reduction)
     std::vector<int> first(n_inst + 1, 0);
     for (int i = 0; i < n_inst; ++i) first[i + 1] = first[i] + c->hI[i].ntile_nodes;
@@ -765,6 +805,7 @@ es_status es_create_batch(const es_config* cfgs, int n_inst, es_ctx** out)
     if (c->d == 2) {
         c->fused_shape = 0;
         c->fused_grid = c->sms * flux2d_occ(c, 0);
+        pick_fused(c);
     }
     cudaError_t e = cudaDeviceSynchronize();
     if (!ok || e != cudaSuccess || !c->w_pad || !c->w_cell || (c->d == 3 && (!c->w_ext || !c->w_col || (!c->mixed && !c->w_xe)))) {
@@ -1116,11 +1157,13 @@ es_status es_autotune(es_ctx* c, const double* JU, const double* J, const double
     // 2D: the fused stage launch in each fused shape against the sum of the best
     // per-direction launches (both in MODE_WRITE); the faster form is kept
     c->fused_shape = -1;
+    c->fused_run = -1;
     c->fused_ms = 0.f;
     drop_run_graph(c);
     if (c->d == 2) {
+        // the small-grid shapes last: they take over the launch, not the reported shape
         float best = 3.0e38f;
-        for (int sh = 0; sh < NFSHAPE; ++sh) {
+        for (int sh = 0; sh < NFSHAPE_ALL; ++sh) {
             const int occ = flux2d_occ(c, sh);
             for (int o = occ; o >= 1 && o >= occ - 1; --o) {
                 FluxLaunch L;
@@ -1149,8 +1192,17 @@ es_status es_autotune(es_ctx* c, const double* JU, const double* J, const double
                     best = ms;
                     c->fused_ms = ms;
                     if (ms < c->flux_ms[0] + c->flux_ms[1]) {
-                        c->fused_shape = sh;
-                        c->fused_grid = grid;
+                        if (sh < NFSHAPE) {
+                            c->fused_shape = sh;
+                            c->fused_grid = grid;
+                        } else {
+                            if (c->fused_shape < 0) {
+                                c->fused_shape = 0;
+                                c->fused_grid = c->sms * flux2d_occ(c, 0);
+                            }
+                            c->fused_run = sh;
+                            c->fused_run_grid = grid;
+                        }
                     }
                 }
             }
@@ -1159,13 +1211,14 @@ es_status es_autotune(es_ctx* c, const double* JU, const double* J, const double
     // mixed 2D: the fused mesh-step launch in each tile shape, after the passes it reads
     // (metrics, CFL and monitor gradients) on the same state; it writes only scratch
     c->jf_ms = 0.f;
+    c->jf_run = -1;
     if (fused_mesh2d(c)) {
         StagePtrs Q = P;
         Q.xdot = nullptr;
         launch_metrics(c, Q, tab, st, true, false, false);
         launch_cfl_grad(c->mixed, c->d, c->N, node_grid(c, c->n_cell), st, c->dI, P, tab, c->w_cell, c->n_cell, c->dS);
         float best = 3.0e38f;
-        for (int sh = 0; sh < NJF_SHAPE; ++sh) {
+        for (int sh = 0; sh < NJF_SHAPE_ALL; ++sh) {
             launch_fused_mesh2d(c, sh, P, tab, st);
             cudaEventRecord(e0, st);
             for (int r = 0; r < reps; ++r) launch_fused_mesh2d(c, sh, P, tab, st);
@@ -1177,7 +1230,8 @@ es_status es_autotune(es_ctx* c, const double* JU, const double* J, const double
             if (ms < best) {
                 best = ms;
                 c->jf_ms = ms;
-                c->jf_shape = sh;
+                if (sh < NJF_SHAPE) c->jf_shape = sh;
+                else c->jf_run = sh;
             }
         }
     }
@@ -1204,6 +1258,7 @@ es_status es_set_mesh_tiles(es_ctx* c, int shape)
     if (!c->mixed || c->d != 2 || shape < 0 || shape >= NJF_SHAPE)
         return fail(c, ES_ERR_ARG, "es_set_mesh_tiles: shape out of range or not a mixed-form 2D context");
     c->jf_shape = shape;
+    c->jf_run = -1;
     c->jf_ms = 0.f;
     drop_run_graph(c);
     return ES_OK;
@@ -1255,6 +1310,7 @@ es_status es_set_fusion(es_ctx* c, int shape, int grid)
     c->fused_shape = shape;
     c->fused_grid = shape >= 0 ? (grid > 0 ? grid : c->sms * flux2d_occ(c, shape)) : 0;
     c->fused_ms = 0.f;
+    c->fused_run = -1;
     drop_run_graph(c);
     return ES_OK;
 }

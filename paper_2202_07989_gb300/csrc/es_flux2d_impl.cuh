@@ -228,8 +228,8 @@ __global__ void __launch_bounds__(FLUX_TPB, (sizeof(R) == 4 ? 3 : 1)) flux2d_ker
 }
 
 // one case per fused tile shape of the table in es_kernels.cuh
-#define ES_FLUX2D_SHAPES(X) X(0) X(1) X(2) X(3) X(4)
-static_assert(NFSHAPE == 5, "ES_FLUX2D_SHAPES lists every fused tile shape");
+#define ES_FLUX2D_SHAPES(X) X(0) X(1) X(2) X(3) X(4) X(5) X(6) X(7)
+static_assert(NFSHAPE_ALL == 8, "ES_FLUX2D_SHAPES lists every fused tile shape");
 
 template <int NS, typename R, int WK>
 void prepare_flux2d()

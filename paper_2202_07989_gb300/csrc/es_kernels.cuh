@@ -15,10 +15,19 @@ constexpr int SHAPE_WT[NSHAPE] = { 4, 4, 2, 8, 8, 16 };
 constexpr int SHAPE_DEFAULT_K0 = 0;    // direction 1: 62 nodes along the line x 4 lines
 constexpr int SHAPE_DEFAULT_KN = 3;    // directions 2, 3: 30 nodes x 8 neighbouring lines (coalesced)
 // fused 2D stage tiles (both directions in one launch): TX x TY output nodes, at most 256
-// interfaces per direction; the autotuner picks one shape, or the per-direction launches
+// interfaces per direction; the autotuner picks one shape, or the per-direction launches.  The
+// shapes from NFSHAPE on are for small grids: a grid of few tiles is bound by the time one tile
+// takes, not by the chip, and a smaller tile takes less.  FSHAPE_COST is the time of one wave of
+// CTAs in each shape relative to 16 x 12 tiles, binary32 and binary64 (launch and metrics pass
+// included, measured on grids of one wave: 16 x 12 21.6 / 176 us, 8 x 8 17.0 / 92, 12 x 8 17.8 /
+// 107, 16 x 8 19.4 / 138 at 64^2 single-species), by which a context that nobody tuned picks
+// its tiles: the least waves x cost (pick_fused in es_api.cu).
 constexpr int NFSHAPE = 5;
-constexpr int FSHAPE_TX[NFSHAPE] = { 16, 12, 14, 24, 20 };
-constexpr int FSHAPE_TY[NFSHAPE] = { 12, 16, 14, 8, 10 };
+constexpr int NFSHAPE_ALL = 8;
+constexpr int FSHAPE_TX[NFSHAPE_ALL] = { 16, 12, 14, 24, 20, 8, 12, 16 };
+constexpr int FSHAPE_TY[NFSHAPE_ALL] = { 12, 16, 14, 8, 10, 8, 8, 8 };
+constexpr double FSHAPE_COST[NFSHAPE_ALL][2] = { { 1.0, 1.0 }, { 1.0, 1.0 }, { 1.0, 1.0 }, { 1.0, 1.0 }, { 1.0, 1.0 },
+                                                 { 0.75, 0.5 }, { 0.8, 0.6 }, { 0.88, 0.78 } };
 constexpr int NODE_TPB = 256;
 
 // launch with programmatic stream serialization (the kernel must begin with pdl_entry())

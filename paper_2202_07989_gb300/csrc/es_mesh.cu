@@ -815,10 +815,19 @@ struct SlotIterN {
 using SlotIter = SlotIterN<NODE_TPB>;
 
 
+// an index at most a few periods outside [0, n) wrapped into it (no integer division: the region of
+// a tile reaches one period at most on all but the smallest grids)
+__device__ __forceinline__ int wrap_near(int g, int n)
+{
+    while (g < 0) g += n;
+    while (g >= n) g -= n;
+    return g;
+}
+
 // whether the (unwrapped) node position (g0, g1) is the first or last node of the grid in a direction
 __device__ __forceinline__ bool grid_edge(int g0, int n0, bool per0, int g1, int n1, bool per1)
 {
-    const int w0 = per0 ? g0 - floordiv_(g0, n0) * n0 : g0, w1 = per1 ? g1 - floordiv_(g1, n1) * n1 : g1;
+    const int w0 = per0 ? wrap_near(g0, n0) : g0, w1 = per1 ? wrap_near(g1, n1) : g1;
     return w0 == 0 || w0 == n0 - 1 || w1 == 0 || w1 == n1 - 1;
 }
 
@@ -893,13 +902,21 @@ __global__ void __launch_bounds__(TPB, 1024 / TPB) jacobi_fused2d_kernel(const I
         // F filter passes (weights (1/2)^(|j|_1 + 2) over the 3 x 3 stencil)
         float* tc_ = ta;
         float* tn_ = tb;
+        // bit s: slot s of this thread is a first or last grid node (at most 9 slots a thread)
+        unsigned int edge_slots = 0;
+        if (pass.edges && F > 0) {
+            unsigned int bit = 1;
+            for (SI sl(RXo); sl.q < NRo; sl.next(), bit <<= 1)
+                if (grid_edge(o0 + sl.a, n0, per0, o1 + sl.b, n1, per1)) edge_slots |= bit;
+        }
         for (int f = 0; f < F; ++f) {
-            for (SI sl(RXo); sl.q < NRo; sl.next()) {
+            unsigned int bit = 1;
+            for (SI sl(RXo); sl.q < NRo; sl.next(), bit <<= 1) {
                 const int q = sl.q, a = sl.a, b = sl.b;
                 const int g0 = o0 + a, g1 = o1 + b;
                 const bool ghost = (!per0 && (g0 < 0 || g0 >= n0)) || (!per1 && (g1 < 0 || g1 >= n1));
                 if (ghost || a == 0 || a == RXo - 1 || b == 0 || b == RYo - 1) continue;
-                const bool edge = pass.edges && grid_edge(g0, n0, per0, g1, n1, per1);
+                const bool edge = (edge_slots & bit) != 0;
                 float acc = 0.0f;
 #pragma unroll
                 for (int j2 = -1; j2 <= 1; ++j2) {
@@ -947,7 +964,7 @@ __global__ void __launch_bounds__(TPB, 1024 / TPB) jacobi_fused2d_kernel(const I
             ya[q] = yb[q] = y0[0];
             ya[NR + q] = yb[NR + q] = y0[1];
             if (ghost) continue;
-            const int w0 = per0 ? g0 - floordiv_(g0, n0) * n0 : g0, w1 = per1 ? g1 - floordiv_(g1, n1) * n1 : g1;
+            const int w0 = per0 ? wrap_near(g0, n0) : g0, w1 = per1 ? wrap_near(g1, n1) : g1;
             const long long c = lin(I, w0, w1, 0);
             const double xc[2] = { P.x[c], P.x[n + c] };
 #pragma unroll
@@ -997,7 +1014,7 @@ __global__ void __launch_bounds__(TPB, 1024 / TPB) jacobi_fused2d_kernel(const I
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
                 const bool wall = k == 0 ? (!per0 && g0 == 0) : (!per1 && g1 == 0);
-                if (pass.edges && (k == 0 ? g0 - floordiv_(g0, n0) * n0 : g1 - floordiv_(g1, n1) * n1) == 0) continue;
+                if (pass.edges && (k == 0 ? wrap_near(g0, n0) : wrap_near(g1, n1)) == 0) continue;
                 if (wall || (k == 0 ? a == 0 : b == 0)) continue;
                 const int qn = q - (k == 0 ? 1 : RX);
 #pragma unroll
@@ -1084,7 +1101,7 @@ size_t jacobi_fused2d_smem(int H, int F, int shape)
     return sizeof(float) * (17 * nr + 2 * nro);
 }
 
-#define JF_KERNELS(X) X(0, 32, 8, 256) X(1, 32, 16, 512) X(2, 24, 16, 512) X(3, 24, 12, 512)
+#define JF_KERNELS(X) X(0, 32, 8, 256) X(1, 32, 16, 512) X(2, 24, 16, 512) X(3, 24, 12, 512) X(4, 16, 8, 512) X(5, 8, 8, 512)
 
 void prepare_mesh()
 {

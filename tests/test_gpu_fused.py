@@ -286,3 +286,38 @@ def test_mesh_sweeps_in_several_launches(bc, mu, nf):
         assert abs(float(dd[0]) - dt_o) <= 5e-6 * dt_o
         assert abs(float(dd[1]) - dtau_o) <= 5e-5 * dtau_o
         assert np.abs(xd.cpu().numpy() - xd_o).max() <= 5e-5 * np.abs(xd_o).max()
+
+
+@pytest.mark.parametrize("form", [0, 1])
+@pytest.mark.parametrize("N,n,weno", [(1, (10, 11), 0), (1, (64, 64), 0), (2, (81, 41), 1), (2, (150, 75), 0), (1, (128, 121), 0)])
+def test_small_grid_tiles_bitwise(form, N, n, weno):
+    """The tiles that an untuned context takes on a small grid (8 x 8, 12 x 8 and 16 x 8, with
+    ragged edges) give the residual and the RK step of the 16 x 12 tiles bit for bit."""
+    torch = need_gpu()
+    pb, JU, J, x, xdot = case(2, N, n, "mixed", es=True, seed=51 + N, jump=True)
+    pb = pb.with_(weno=weno)
+    a, b = _ctx(pb, form), _ctx(pb, form)
+    assert a.es_get_fusion()[:3] == (0, 16, 12)
+    b.es_set_fusion(0)
+    G = [to_dev(t, torch) for t in (JU, J, x, xdot)]
+    assert _same(a.es_rhs(*G), b.es_rhs(*G))
+    dt = torch.tensor([0.3 * Oracle(pb).cfl_dt(JU, J, x)], dtype=torch.float64, device="cuda")
+    A, B = [t.clone() for t in G[:3]], [t.clone() for t in G[:3]]
+    a.es_rk_step(*A, G[3], dt)
+    b.es_rk_step(*B, G[3], dt)
+    assert _same(A, B)
+
+
+@pytest.mark.parametrize("N,n,mu,nf", [(1, (10, 11), 5, 3), (1, (64, 64), 10, 3), (2, (129, 65), 8, 4), (2, (200, 199), 5, 3), (1, (33, 300), 1, 0)])
+@pytest.mark.parametrize("bc", ["periodic", "mixed"])
+def test_untuned_mesh_tiles_bitwise(bc, N, n, mu, nf):
+    """The mesh tiles that an untuned context takes (8 x 8 and 16 x 8 on small grids) give the mesh
+    velocity and Delta t / Delta tau of the 32 x 8 tiles bit for bit."""
+    torch = need_gpu()
+    pb, JU, J, x, _ = case(2, N, n, bc, es=True, seed=61 + N, jump=True)
+    pb = pb.with_(mu=mu, nf=nf)
+    a, b = _ctx(pb, 1), _ctx(pb, 1)
+    assert a.es_get_mesh_tiles()[:3] == (0, 32, 8)
+    b.es_set_mesh_tiles(0)
+    G = [to_dev(t, torch) for t in (JU, J, x)]
+    assert _same(a.mesh_redistribute(*G), b.mesh_redistribute(*G))
