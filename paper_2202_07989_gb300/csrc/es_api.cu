@@ -181,6 +181,9 @@ Inst make_inst(const es_config& g)
     }
     I.es = g.es;
     for (int q = 0; q < 3; ++q) I.chi[q] = g.chi[q];
+    I.chi_unit = std::fabs(g.chi[0] + g.chi[1] + g.chi[2] - 1.0) <= 1.0e-15;
+    I.sq21 = std::sqrt(I.Rs[1] / I.Rs[0]);
+    I.sq12 = std::sqrt(I.Rs[0] / I.Rs[1]);
     I.weno_eps = g.weno_eps;
     I.cfl = g.cfl;
     I.n_sigma = g.n_sigma;

@@ -57,6 +57,8 @@ struct Inst {
     float f_ichi3;            // 1 / chi_3 of WENO-MR
     double mc[3][3];          // (1/2) alpha_m / dxi_k: delta_k of a coordinate divided by dxi_k
     int w;                    // EC flux order 2w
+    int chi_unit;             // the WENO-MR linear weights sum to one
+    double sq21, sq12;        // (R_2 / R_1)^(1/2) and its reciprocal (two species)
     double ecw[3];            // alpha_m of order 2w (zero for m > w): the EC pair sum and delta_k
     double gcw[3];            // the GCL stencil: (1/2) sum_{m >= j+1} alpha_m for node pairs j = 0..2
     float f_ecw[3], f_gcw[3]; // binary32 copies

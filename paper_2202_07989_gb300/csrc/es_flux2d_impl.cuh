@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(FLUX_TPB, (sizeof(R) == 4 ? 3 : 1)) flux2d_ker
                     const long long id = k == 0 ? lin(I, gi, j, 0) : lin(I, i, gi, 0);
                     const R inv = Ar<R>::rcp(to_r<R>(P.J[id]));
 #pragma unroll
-                    for (int q = 0; q < NC; ++q) U[q] = to_r<R>(P.JU[q * ncell + id]) * inv;
+                    for (int q = 0; q < NC; ++q) U[q] = mulr(to_r<R>(P.JU[q * ncell + id]), inv);
                     if (tmap == 1) U[NS + k] = -U[NS + k];
                 }
             }

@@ -35,37 +35,47 @@ struct Ar<double> {
     static __device__ __forceinline__ double lg(double x) { return log(x); }
     static __device__ __forceinline__ double sq(double x) { return sqrt(x); }
     static __device__ __forceinline__ double ab(double x) { return fabs(x); }
-    // {a}^ln: [[a]]/[[ln a]], Ismail-Roe series when ((b-a)/(b+a))^2 < 1e-4
-    static __device__ __forceinline__ double lmean(double a, double b, double la, double lb)
+    // |dd| < s / 128, on the high words: no FP64 comparison (it would issue on the FP64 pipe).
+    // Series and quotient agree to round-off around this threshold, so its last bits are free.
+    static __device__ __forceinline__ bool small_jump(double dd, double s)
     {
-        double s = a + b, dd = b - a;
-        if (fabs(dd) < 0.01 * s) {
-            double f = dd / s, u = f * f;
-            return 0.5 * s * (1.0 - u * (1.0 / 3.0 + u * (4.0 / 45.0 + u * (44.0 / 945.0))));
+        return (__double2hiint(dd) & 0x7fffffff) < __double2hiint(s) - (7 << 20);
+    }
+    // {a}^ln: [[a]]/[[ln a]], Ismail-Roe series at small jumps; is = 1/(a + b)
+    static __device__ __forceinline__ double lmean_is(double a, double b, double is, double la, double lb)
+    {
+        const double s = a + b, dd = b - a;
+        if (small_jump(dd, s)) {
+            const double f = dd * is, u = f * f;
+            return __dmul_rn(0.5 * s, fma(-u, fma(u, fma(u, 44.0 / 945.0, 4.0 / 45.0), 1.0 / 3.0), 1.0));
         }
         return dd / (lb - la);
     }
-    // 1/{a}^ln given is = 1/(a + b)
+    // 1/{a}^ln
     static __device__ __forceinline__ double inv_lmean(double a, double b, double la, double lb, double is)
     {
-        double dd = b - a;
-        if (fabs(dd) < 0.01 * (a + b)) {
-            double f = dd * is, u = f * f;
-            return 2.0 * is * (1.0 + u * (1.0 / 3.0 + u * (1.0 / 5.0 + u * (1.0 / 7.0))));
+        const double dd = b - a;
+        if (small_jump(dd, a + b)) {
+            const double f = dd * is, u = f * f;
+            return __dmul_rn(2.0 * is, fma(u, fma(u, fma(u, 1.0 / 7.0, 1.0 / 5.0), 1.0 / 3.0), 1.0));
         }
         return (lb - la) / dd;
     }
     // the same with the logarithms formed only in their branch
+    static __device__ __forceinline__ double lmean_is(double a, double b, double is)
+    {
+        if (small_jump(b - a, a + b)) return lmean_is(a, b, is, 0.0, 0.0);
+        return (b - a) / (lg(b) - lg(a));
+    }
     static __device__ __forceinline__ double lmean(double a, double b)
     {
-        double s = a + b, dd = b - a;
-        if (fabs(dd) < 0.01 * s) return lmean(a, b, 0.0, 0.0);
-        return dd / (lg(b) - lg(a));
+        if (small_jump(b - a, a + b)) return lmean_is(a, b, 1.0 / (a + b), 0.0, 0.0);
+        return (b - a) / (lg(b) - lg(a));
     }
     static __device__ __forceinline__ double inv_lmean(double a, double b, double is)
     {
-        double dd = b - a;
-        if (fabs(dd) < 0.01 * (a + b)) return inv_lmean(a, b, 0.0, 0.0, is);
+        const double dd = b - a;
+        if (small_jump(dd, a + b)) return inv_lmean(a, b, 0.0, 0.0, is);
         return (lg(b) - lg(a)) / dd;
     }
 };
@@ -118,6 +128,16 @@ struct Ar<float> {
     }
 };
 
+// a b + c d and a b + c in one fixed evaluation order in binary64 (the compiler picks which
+// product of a sum it fuses, and may pick differently in each tile shape's kernel, whose results
+// are to be equal bit for bit); binary32 keeps the plain expression
+__device__ __forceinline__ double dot2(double a, double b, double c, double d) { return fma(c, d, __dmul_rn(a, b)); }
+__device__ __forceinline__ float dot2(float a, float b, float c, float d) { return a * b + c * d; }
+__device__ __forceinline__ double mad(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ float mad(float a, float b, float c) { return a * b + c; }
+__device__ __forceinline__ double mulr(double a, double b) { return __dmul_rn(a, b); }     // never fused
+__device__ __forceinline__ float mulr(float a, float b) { return a * b; }
+
 // Sign band of the sign matrix Y (Sec. 3.4): a jump [[W_m]] no larger than delta times
 // its round-off scale ||r_m|| (||V_i|| + ||V_i+1||) has no reliable sign and counts as
 // zero, like an exactly zero jump (Y = 0 keeps the ES sign property).
@@ -159,6 +179,60 @@ __device__ __forceinline__ R weno_mr(R w0, R w1, R w2, R w3, R w4, R c1, R c2, R
         R o1 = c1 * (R(1) + Ar<R>::dv(tau, e1)), o2 = c2 * (R(1) + Ar<R>::dv(tau, e2)), o3 = c3 * (R(1) + Ar<R>::dv(tau, e3));
         return Ar<R>::dv(o1 * h1 + o2 * h2 + o3 * h3c, o1 + o2 + o3);
     }
+}
+
+// weno_mr of the FP64 form out of line, for linear weights that do not sum to one
+static __device__ __noinline__ double weno_mr_any(double w0, double w1, double w2, double w3, double w4, double c1, double c2,
+                                                  double c3, double eps)
+{
+    return weno_mr<double>(w0, w1, w2, w3, w4, c1, c2, c3, eps);
+}
+
+// the smaller of two non-negative values, compared on the integer pipe
+__device__ __forceinline__ double min_pos(double a, double b)
+{
+    return __double_as_longlong(a) < __double_as_longlong(b) ? a : b;
+}
+
+// WENO-MR (Appendix A) of the FP64 form from the node differences D_m = W_{j-1+m} - W_{j-2+m}
+// (m = 0..3): the value at x_{j+1/2} is W_j + num / den, for linear weights that sum to one.
+// The indicators, candidate values and weights of weno_mr, written in s = D1 + D2, e = D2 - D1,
+// t = D0 + D3, u = D3 - D0 and cleared of the common denominator: t_1 = (7s - t)/12, t_2 =
+// (163e - 11u)/260, b_4 = (t - s)/12, b_5 = (u - 3e)/24, h_2 - W_j = s/4 + e/12, h_3 - W_j =
+// (-2 D0 + 11 D1 + 24 D2 - 3 D3)/60.  All differences of W, so nothing cancels against W itself.
+// Why: the FP64 form is bound by its pipe, and this takes about 50 FP64 instructions and no
+// division where weno_mr takes about 80 with one; W^+ mirrors to the same function of the
+// negated differences, so the jump needs one division for both (weno_mr_jump).
+__device__ __forceinline__ void weno_mr_corr(double D0, double D1, double D2, double D3, double q1, double q2, double c1,
+                                             double c2, double c3, double eps, double& num, double& den)
+{
+    const double s = D1 + D2, e = D2 - D1, t = D0 + D3, u = D3 - D0, h = 0.5 * s;
+    const double E1 = eps + min_pos(q1, q2);
+    const double E2 = fma((13.0 / 12.0) * e, e, fma(h, h, eps));
+    const double A = fma(7.0, s, -t), P = t - s, B = fma(-11.0 / 163.0, u, e), r = fma(-3.0, e, u);
+    const double E3 = fma((1.0 / 144.0) * A, A, fma((781.0 / 2880.0) * P, P, fma((26569.0 / 15600.0) * B, B,
+                      fma((1421461.0 / 1310400.0) * r, r, eps))));
+    const double x = fabs(E3 - E1) + fabs(E3 - E2), X = x * x;     // tau = X / 4
+    const double f1 = fma(0.25, X, E1), f2 = fma(0.25, X, E2), f3 = fma(0.25, X, E3);
+    const double h2 = fma(1.0 / 12.0, e, 0.5 * h);
+    const double h3 = fma(24.0 / 60.0, D2, fma(11.0 / 60.0, D1, fma(-3.0 / 60.0, D3, (-2.0 / 60.0) * D0)));
+    const double o1 = __dmul_rn(c1 * f1, E2 * E3), o2 = __dmul_rn(c2 * f2, E1 * E3), o3 = __dmul_rn(f3, E1 * E2);
+    den = fma(c3, o3, o1 + o2);
+    num = fma(o2, h2, __dmul_rn(o3, fma(-c2, h2, h3)));
+}
+
+// [[W]]^WENO-MR at the interface from the five node differences D_0..D_4 of its stencil
+__device__ __forceinline__ double weno_mr_jump(const double* D, double c1, double c2, double c3, double eps)
+{
+    const double q1 = __dmul_rn(D[1], D[1]), q2 = __dmul_rn(D[2], D[2]), q3 = __dmul_rn(D[3], D[3]);
+    double nm, dm, np, dp;
+    weno_mr_corr(D[0], D[1], D[2], D[3], q1, q2, c1, c2, c3, eps, nm, dm);
+    weno_mr_corr(D[4], D[3], D[2], D[1], q3, q2, c1, c2, c3, eps, np, dp);
+    const double dd = dm * dp;
+    // one division while the product of the denominators is well inside the range
+    const unsigned int hi = (unsigned int)__double2hiint(dd);
+    if (hi - (100u << 20) < (1846u << 20)) return D[2] - fma(nm, dp, __dmul_rn(np, dm)) / dd;
+    return D[2] - nm / dm - np / dp;
 }
 
 // binary32 pairs: two independent evaluations in the two lanes of Blackwell's paired FP32
@@ -286,8 +360,14 @@ __device__ __forceinline__ void node_fields(const Inst& I, const R* U, R* nr, in
     R v[D], v2 = R(0);
 #pragma unroll
     for (int m = 0; m < D; ++m) { v[m] = U[NS + m] * irho; v2 += v[m] * v[m]; }
-    R cvr = Cst<R>::cv(I, 0) * U[0] + (NS == 2 ? Cst<R>::cv(I, 1) * U[1] : R(0));
-    R rhoe_p = U[NS + D] - R(0.5) * rho * v2 - Cst<R>::pinf(I);
+    R cvr, rhoe_p;
+    if constexpr (std::is_same<R, double>::value) {
+        cvr = NS == 2 ? dot2(I.cv[0], U[0], I.cv[1], U[1]) : I.cv[0] * U[0];
+        rhoe_p = fma(-0.5 * rho, v2, U[NS + D]) - I.pinf_tot;
+    } else {
+        cvr = Cst<R>::cv(I, 0) * U[0] + (NS == 2 ? Cst<R>::cv(I, 1) * U[1] : R(0));
+        rhoe_p = U[NS + D] - R(0.5) * rho * v2 - Cst<R>::pinf(I);
+    }
     R beta = cvr * Ar<R>::rcp(rhoe_p);
     bool bad = !(rhoe_p > R(0)) || !(U[0] > R(0)) || (NS == 2 && !(U[1] > R(0)));
     if (bad) {
@@ -310,20 +390,31 @@ __device__ __forceinline__ void node_fields(const Inst& I, const R* U, R* nr, in
     nr[Y::B * NN + node] = beta;
     nr[Y::LB * NN + node] = lb;
     if (NS == 2) {
-        R T = Ar<R>::rcp(beta);
-        R rr = Cst<R>::Rs(I, 0) * U[0] + Cst<R>::Rs(I, 1) * U[1];
-        nr[(Y::X + 0) * NN + node] = rr * T - Cst<R>::pinf(I);                 // p
+        R T;
+        // (FP64: one reciprocal serves T and Gamma_mix)
+        R icvr = Ar<R>::rcp(cvr);
+        if constexpr (std::is_same<R, double>::value) T = bad ? R(1) : rhoe_p * icvr;
+        else T = Ar<R>::rcp(beta);
+        R rr = dot2(Cst<R>::Rs(I, 0), U[0], Cst<R>::Rs(I, 1), U[1]);
+        nr[(Y::X + 0) * NN + node] = mad(rr, T, -Cst<R>::pinf(I));                 // p
         nr[(Y::X + 1) * NN + node] = rho;                                    // rho
-        nr[(Y::X + 2) * NN + node] = Ar<R>::lg(bad ? R(1) : rho);           // ln rho
+        // ln rho (the FP64 form takes it only in the branch of the log mean that needs it)
+        if constexpr (!std::is_same<R, double>::value) nr[(Y::X + 2) * NN + node] = Ar<R>::lg(bad ? R(1) : rho);
         nr[(Y::X + 3) * NN + node] = rr * irho;                              // R_mix
-        nr[(Y::X + 4) * NN + node] = (Cst<R>::cvG(I, 0) * U[0] + Cst<R>::cvG(I, 1) * U[1]) * Ar<R>::rcp(cvr);  // Gamma_mix
+        nr[(Y::X + 4) * NN + node] = dot2(Cst<R>::cvG(I, 0), U[0], Cst<R>::cvG(I, 1), U[1]) * icvr;  // Gamma_mix
     }
     }
     // entropy variables V_l = c_{v,l} ln beta + R_l ln rho_l - |v|^2 beta/2 + c_{v,l} Gamma_l
-    R hv = R(0.5) * v2 * beta;
     R Vn[NC];
-    Vn[0] = Cst<R>::cv(I, 0) * lb + Cst<R>::Rs(I, 0) * lr0 - hv + Cst<R>::cvG(I, 0);
-    if (NS == 2) Vn[1] = Cst<R>::cv(I, 1) * lb + Cst<R>::Rs(I, 1) * lr1 - hv + Cst<R>::cvG(I, 1);
+    if constexpr (std::is_same<R, double>::value) {
+        const double hv = __dmul_rn(0.5 * v2, beta);
+        Vn[0] = dot2(I.cv[0], lb, I.Rs[0], lr0) - hv + I.cvG[0];
+        if (NS == 2) Vn[1] = dot2(I.cv[1], lb, I.Rs[1], lr1) - hv + I.cvG[1];
+    } else {
+        R hv = R(0.5) * v2 * beta;
+        Vn[0] = Cst<R>::cv(I, 0) * lb + Cst<R>::Rs(I, 0) * lr0 - hv + Cst<R>::cvG(I, 0);
+        if (NS == 2) Vn[1] = Cst<R>::cv(I, 1) * lb + Cst<R>::Rs(I, 1) * lr1 - hv + Cst<R>::cvG(I, 1);
+    }
 #pragma unroll
     for (int m = 0; m < D; ++m) Vn[NS + m] = v[m] * beta;
     Vn[NS + D] = -beta;
@@ -331,6 +422,71 @@ __device__ __forceinline__ void node_fields(const Inst& I, const R* U, R* nr, in
 #pragma unroll
     for (int q = 0; q < NC; ++q) { nr[(Y::VV + q) * NN + node] = Vn[q]; vn += Vn[q] * Vn[q]; }
     if constexpr (!Y::COMPACT) nr[Y::VN * NN + node] = Ar<R>::sq(vn);
+}
+
+// pair_flux in the FP64 form, with fewer FP64 instructions: the reciprocals of the two-point sums
+// of every log mean come from one division, and the kinetic terms of E', sum_m ({v_m}^2 -
+// {v_m^2}/2), are half the dot product of the two velocities
+template <int D, int NS>
+__device__ __forceinline__ void pair_flux64(const Inst& I, const double* nr, int NN, int mr, int l, int rr, double* pf,
+                                            int NP, int t, double* cm, int NI, int ci)
+{
+    using Y = Lay<D, NS>;
+    using A = Ar<double>;
+    constexpr int NC = Y::NC;
+    const double mt = 0.5 * (nr[mr * NN + l] + nr[mr * NN + rr]);
+    double mx[D], vb[D], ut = mt, vlr = 0.0;
+#pragma unroll
+    for (int j = 0; j < D; ++j) {
+        mx[j] = 0.5 * (nr[(mr + 1 + j) * NN + l] + nr[(mr + 1 + j) * NN + rr]);
+        const double vl = nr[(Y::V + j) * NN + l], vr = nr[(Y::V + j) * NN + rr];
+        vb[j] = 0.5 * (vl + vr);
+        vlr = j == 0 ? vl * vr : fma(vl, vr, vlr);
+        ut = fma(mx[j], vb[j], ut);
+    }
+    double al[NS], ar[NS], bl, br;
+#pragma unroll
+    for (int q = 0; q < NS; ++q) { al[q] = nr[(Y::RHO + q) * NN + l]; ar[q] = nr[(Y::RHO + q) * NN + rr]; }
+    if constexpr (Y::COMPACT) { bl = -nr[(Y::VV + NC - 1) * NN + l]; br = -nr[(Y::VV + NC - 1) * NN + rr]; }
+    else { bl = nr[Y::B * NN + l]; br = nr[Y::B * NN + rr]; }
+    // 1 / (rho_l sums) and 1 / (beta sum)
+    const double s0 = al[0] + ar[0], sb = bl + br;
+    double is, ir[NS];
+    if constexpr (NS == 1) {
+        const double r = 1.0 / (s0 * sb);
+        is = r * s0;
+        ir[0] = r * sb;
+    } else {
+        const double s1 = al[1] + ar[1], p = s0 * s1, r = 1.0 / (p * sb), rb = r * sb;
+        is = r * p;
+        ir[0] = rb * s1;
+        ir[1] = rb * s0;
+    }
+    double lr[NS], rt = 0.0, rra = 0.0;
+#pragma unroll
+    for (int q = 0; q < NS; ++q) {
+        if constexpr (Y::COMPACT) lr[q] = A::lmean_is(al[q], ar[q], ir[q]);
+        else lr[q] = A::lmean_is(al[q], ar[q], ir[q], nr[(Y::LRHO + q) * NN + l], nr[(Y::LRHO + q) * NN + rr]);
+        rt = q == 0 ? lr[q] : rt + lr[q];
+        rra = q == 0 ? I.Rs[q] * (al[q] + ar[q]) : fma(I.Rs[q], al[q] + ar[q], rra);
+    }
+    double ilb;
+    if constexpr (Y::COMPACT) ilb = A::inv_lmean(bl, br, is);
+    else ilb = A::inv_lmean(bl, br, nr[Y::LB * NN + l], nr[Y::LB * NN + rr], is);
+    const double Pp = rra * is;                        // sum R_l {rho_l} / {beta}
+    double cl = I.cv[0] * lr[0];
+    if constexpr (NS == 2) cl = fma(I.cv[1], lr[1], cl);
+    const double Ep = fma(cl, ilb, 0.5 * rt * vlr), utr = ut * rt;
+#pragma unroll
+    for (int q = 0; q < NS; ++q) pf[q * NP + t] = ut * lr[q];
+#pragma unroll
+    for (int j = 0; j < D; ++j) pf[(NS + j) * NP + t] = fma(utr, vb[j], mx[j] * Pp);
+    pf[(NS + D) * NP + t] = fma(ut, Ep, (ut - mt) * Pp);
+    if (ci >= 0) {
+#pragma unroll
+        for (int q = 0; q < NS; ++q) cm[q * NI + ci] = lr[q];
+        cm[NS * NI + ci] = ilb;
+    }
 }
 
 // Phase 2 of one pair (l, r) of nodes: the contracted two-point flux of every field into
@@ -343,6 +499,9 @@ __device__ __forceinline__ void pair_flux(const Inst& I, const R* nr, int NN, in
 {
     using Y = Lay<D, NS>;
     constexpr int NC = Y::NC;
+    if constexpr (std::is_same<R, double>::value) {
+        pair_flux64<D, NS>(I, nr, NN, mr, l, rr, pf, NP, t, cm, NI, ci);
+    } else {
     R mt = R(0.5) * (nr[mr * NN + l] + nr[mr * NN + rr]);
     R mx[D], vb[D];
     R ut = mt, v2b = R(0), vbsq = R(0);
@@ -391,6 +550,7 @@ __device__ __forceinline__ void pair_flux(const Inst& I, const R* nr, int NN, in
         for (int q = 0; q < NS; ++q) cm[q * NI + ci] = lr[q];
         cm[NS * NI + ci] = ilb;
     }
+    }
 }
 
 // Phase 3 of one interface i+1/2 of a line.  nb points at field 0 of node i-2 of the
@@ -414,19 +574,19 @@ __device__ __forceinline__ void iface_flux(const Inst& I, const R* nb, int NN, i
 #pragma unroll
     for (int q = 0; q < NC; ++q) {
         const R* pq = pf + q * NP;
-        fl[q * NI + f] = a1 * pq[p1] + a2 * (pq[p2] + pq[p2 + ps]) + a3 * (pq[p3] + pq[p3 + ps] + pq[p3 + 2 * ps]);
+        fl[q * NI + f] = mad(a3, pq[p3] + pq[p3 + ps] + pq[p3 + 2 * ps], dot2(a1, pq[p1], a2, pq[p2] + pq[p2 + ps]));
     }
     // GCL flux of (J xi_k/t, J xi_k/x_j): stencil (1, -8, 37, 37, -8, 1)/60 for w = 3
     const double c0 = I.gcw[0], c1 = I.gcw[1], c2 = I.gcw[2];
-    const double Gt = c0 * (m64[2 * ms] + m64[3 * ms]) + c1 * (m64[ms] + m64[4 * ms]) + c2 * (m64[0] + m64[5 * ms]);
+    const double Gt = mad(c2, m64[0] + m64[5 * ms], dot2(c0, m64[2 * ms] + m64[3 * ms], c1, m64[ms] + m64[4 * ms]));
     gt[f] = Gt;
     if (I.es) {
         R Gx[D], L2 = R(0);
 #pragma unroll
         for (int j = 0; j < D; ++j) {
             const int fj = mr + 1 + j;
-            Gx[j] = Cst<R>::gcw(I, 0) * (NR(fj, 2) + NR(fj, 3)) + Cst<R>::gcw(I, 1) * (NR(fj, 1) + NR(fj, 4)) +
-                    Cst<R>::gcw(I, 2) * (NR(fj, 0) + NR(fj, 5));
+            Gx[j] = mad(Cst<R>::gcw(I, 2), NR(fj, 0) + NR(fj, 5), dot2(Cst<R>::gcw(I, 0), NR(fj, 2) + NR(fj, 3),
+                                                                       Cst<R>::gcw(I, 1), NR(fj, 1) + NR(fj, 4)));
             L2 += Gx[j] * Gx[j];
         }
         R Ln = Ar<R>::sq(L2), iL = Ar<R>::rcp(Ln);
@@ -439,7 +599,7 @@ __device__ __forceinline__ void iface_flux(const Inst& I, const R* nb, int NN, i
             T[0][0] = n[0]; T[0][1] = n[1];
             T[1][0] = -n[1]; T[1][1] = n[0];
         } else {
-            R rr2 = n[0] * n[0] + n[1] * n[1];
+            R rr2 = dot2(n[0], n[0], n[1], n[1]);
             R rq = Ar<R>::sq(rr2);
             R ct = R(1), st = R(0);
             if (rq > R(0)) { R irq = Ar<R>::rcp(rq); ct = n[0] * irq; st = n[1] * irq; }
@@ -468,7 +628,7 @@ __device__ __forceinline__ void iface_flux(const Inst& I, const R* nb, int NN, i
             const R G = Cst<R>::gamma(I, 0), Rg = Cst<R>::Rs(I, 0), cv = Cst<R>::cv(I, 0);
             const R rb = lr_c[0];
             cb = Ar<R>::sq(Rg * G * Tb);
-            H = G * cv * Tb + R(0.5) * vv;
+            H = mad(G * cv, Tb, R(0.5) * vv);
             sa = Ar<R>::sq(rb * Ar<R>::rcp(R(2) * G * Rg));
             se = Ar<R>::sq(rb * Ar<R>::rcp(cv * G));
             ssh = Ar<R>::sq(rb * Tb);
@@ -479,12 +639,12 @@ __device__ __forceinline__ void iface_flux(const Inst& I, const R* nb, int NN, i
             for (int c = 0; c < 2; ++c) {
                 if constexpr (Y::COMPACT) {
                     const R u0 = NR(Y::RHO, 2 + c), u1 = NR(Y::RHO + 1, 2 + c), beta = -NR(Y::VV + NC - 1, 2 + c);
-                    const R rr = Cst<R>::Rs(I, 0) * u0 + Cst<R>::Rs(I, 1) * u1;
-                    const R cvr = Cst<R>::cv(I, 0) * u0 + Cst<R>::cv(I, 1) * u1;
+                    const R rr = dot2(Cst<R>::Rs(I, 0), u0, Cst<R>::Rs(I, 1), u1);
+                    const R cvr = dot2(Cst<R>::cv(I, 0), u0, Cst<R>::cv(I, 1), u1);
                     xr[c] = u0 + u1;
                     xR[c] = rr * Ar<R>::rcp(xr[c]);
-                    xG[c] = (Cst<R>::cvG(I, 0) * u0 + Cst<R>::cvG(I, 1) * u1) * Ar<R>::rcp(cvr);
-                    xp[c] = rr * Ar<R>::rcp(beta) - Cst<R>::pinf(I);
+                    xG[c] = dot2(Cst<R>::cvG(I, 0), u0, Cst<R>::cvG(I, 1), u1) * Ar<R>::rcp(cvr);
+                    xp[c] = mad(rr, Ar<R>::rcp(beta), -Cst<R>::pinf(I));
                 } else {
                     xp[c] = NR(Y::X + 0, 2 + c);
                     xr[c] = NR(Y::X + 1, 2 + c);
@@ -494,17 +654,31 @@ __device__ __forceinline__ void iface_flux(const Inst& I, const R* nb, int NN, i
                 }
             }
             R rb;
-            if constexpr (Y::COMPACT) rb = Ar<R>::lmean(xr[0], xr[1]);
+            if constexpr (Y::COMPACT || std::is_same<R, double>::value) rb = Ar<R>::lmean(xr[0], xr[1]);
             else rb = Ar<R>::lmean(xr[0], xr[1], xl[0], xl[1]);
             const R Rb = R(0.5) * (xR[0] + xR[1]);
             const R Gb = R(0.5) * (xG[0] + xG[1]);
             const R pb = R(0.5) * (xp[0] + xp[1]);
-            R rh = pb + Cst<R>::pinf(I) + (Cst<R>::cv(I, 0) * lr_c[0] + Cst<R>::cv(I, 1) * lr_c[1]) * Tb;
+            R rh = mad(dot2(Cst<R>::cv(I, 0), lr_c[0], Cst<R>::cv(I, 1), lr_c[1]), Tb, pb + Cst<R>::pinf(I));
             R irb = Ar<R>::rcp(rb);
             Y1 = lr_c[0] * irb;
             Y2 = lr_c[1] * irb;
-            H = rh * irb + R(0.5) * vv;
+            H = mad(rh, irb, R(0.5) * vv);
             cb = Ar<R>::sq(Rb * Gb * Tb);
+            if constexpr (std::is_same<R, double>::value) {
+                // the same scalings with shared roots and reciprocals: sqrt(rho / (Gamma R)), times
+                // sqrt(Y1 Y2 Gamma) in one root, and (Gamma - 1)^(1/2), 1/(Gamma - 1) from one rsqrt
+                const double iGR = 1.0 / (Gb * Rb), rg = rb * iGR, gm = Gb - 1.0, ig = rsqrt(gm), igm = ig * ig;
+                const double pre = sqrt(rg), psy = sqrt(rg * (Y1 * Y2) * Gb), psg = pre * (gm * ig);
+                sa = pre * 0.70710678118654752440;
+                ssh = sqrt(rb * Tb);
+                D11 = -psy * I.sq21;
+                D21 = psy * I.sq12;
+                D12 = psg * Y1;
+                D22 = psg * Y2;
+                e1 = fma(-(I.cv[0] + I.Rs[0] - Gb * I.cv[0]) * Tb, igm, 0.5 * vv);
+                e2 = fma(-(I.cv[1] + I.Rs[1] - Gb * I.cv[1]) * Tb, igm, 0.5 * vv);
+            } else {
             const R pre = Ar<R>::sq(rb * Ar<R>::rcp(Gb * Rb));
             sa = pre * R(0.70710678118654752440);
             ssh = Ar<R>::sq(rb * Tb);
@@ -517,8 +691,9 @@ __device__ __forceinline__ void iface_flux(const Inst& I, const R* nb, int NN, i
             R igm = Ar<R>::rcp(Gb - R(1));
             e1 = R(0.5) * vv - (Cst<R>::cv(I, 0) + R1 - Gb * Cst<R>::cv(I, 0)) * Tb * igm;
             e2 = R(0.5) * vv - (Cst<R>::cv(I, 1) + R2 - Gb * Cst<R>::cv(I, 1)) * Tb * igm;
+            }
         }
-        const R lam = Ar<R>::ab(to_r<R>(Gt) + Ln * vh[0]) + Ln * cb;
+        const R lam = mad(Ln, cb, Ar<R>::ab(mad(Ln, vh[0], to_r<R>(Gt))));
         // round-off band of [[W_m]]: delta ||r_m|| (||V_i|| + ||V_i+1||)
         R nvb;
         if constexpr (Y::COMPACT) nvb = vnorm<NC, Y::VV, R>(nb + 2 * ns, NN) + vnorm<NC, Y::VV, R>(nb + 3 * ns, NN);
@@ -528,6 +703,21 @@ __device__ __forceinline__ void iface_flux(const Inst& I, const R* nb, int NN, i
         R Fd[NC];
 #pragma unroll
         for (int q = 0; q < NC; ++q) Fd[q] = R(0);
+        // FP64 WENO-MR works on the node differences of the entropy variables
+        constexpr bool DIFF = std::is_same<R, double>::value && WK == 0;
+        R dV[DIFF ? NC : 1][5];
+        if constexpr (DIFF) {
+#pragma unroll
+            for (int q = 0; q < NC; ++q) {
+                R lo = NR(Y::VV + q, 0);
+#pragma unroll
+                for (int j = 0; j < 5; ++j) {
+                    const R up = NR(Y::VV + q, j + 1);
+                    dV[q][j] = up - lo;
+                    lo = up;
+                }
+            }
+        }
         // the two acoustic columns first, so that their averages are dead for the others.  The
         // 3D two-species tiles keep the loop rolled: unrolled it spills at the 64 registers of 4
         // blocks per SM (800 bytes of spill loads against 212), and rolled it ran the Example 5.11
@@ -546,7 +736,7 @@ __device__ __forceinline__ void iface_flux(const Inst& I, const R* nb, int NN, i
 #pragma unroll
                 for (int j = 0; j < D; ++j) rc[NS + j] = vh[j];
                 rc[NS] += sg * cb;
-                rc[NS + D] = H + sg * cb * vh[0];
+                rc[NS + D] = mad(sg * cb, vh[0], H);
 #pragma unroll
                 for (int q = 0; q < NC; ++q) rc[q] *= sa;
             } else if (col <= NS) {
@@ -561,7 +751,7 @@ __device__ __forceinline__ void iface_flux(const Inst& I, const R* nb, int NN, i
                     rc[1] = db;
 #pragma unroll
                     for (int j = 0; j < D; ++j) rc[2 + j] = (da + db) * vh[j];
-                    rc[2 + D] = da * e1 + db * e2;
+                    rc[2 + D] = dot2(da, e1, db, e2);
                 }
             } else {
                 const int mm = col - NS;      // shear: rotated velocity component mm (1..D-1)
@@ -584,6 +774,46 @@ __device__ __forceinline__ void iface_flux(const Inst& I, const R* nb, int NN, i
 #pragma unroll
             for (int j = 0; j < D; ++j) rc[NS + j] = ru[j];
             // scaled entropy variables W_j = r_col . V_j at the six nodes, then W^- and W^+
+            if constexpr (DIFF) {
+                // (a shear column has no species components)
+                const int q0 = col > NS && col < NC - 1 ? NS : 0;
+                R Dw[5], rn = R(0);
+#pragma unroll
+                for (int j = 0; j < 5; ++j) Dw[j] = R(0);
+#pragma unroll
+                for (int q = 0; q < NC; ++q) {
+                    if (q < q0) continue;
+                    rn = q == q0 ? rc[q] * rc[q] : fma(rc[q], rc[q], rn);
+#pragma unroll
+                    for (int j = 0; j < 5; ++j) Dw[j] = q == q0 ? rc[q] * dV[q][j] : fma(rc[q], dV[q][j], Dw[j]);
+                }
+                // [[W]] beyond the band and of the sign of [[W]]^WENO-MR, decided on the integer pipe
+                const R jp = Dw[2];
+                if (!(__double_as_longlong(jp * jp) > __double_as_longlong(band2 * rn))) continue;
+                R jw;
+                if (I.chi_unit) {
+                    jw = weno_mr_jump(Dw, ch1, ch2, ch3, eps);
+                } else {
+                    // linear weights that do not sum to one weigh W itself, not its differences
+                    R wv[6];
+#pragma unroll
+                    for (int j = 0; j < 6; ++j) {
+                        R s_ = R(0);
+#pragma unroll
+                        for (int q = 0; q < NC; ++q) s_ += rc[q] * NR(Y::VV + q, j);
+                        wv[j] = s_;
+                    }
+                    jw = weno_mr_any(wv[5], wv[4], wv[3], wv[2], wv[1], ch1, ch2, ch3, eps) -
+                         weno_mr_any(wv[0], wv[1], wv[2], wv[3], wv[4], ch1, ch2, ch3, eps);
+                }
+                const int sj = __double2hiint(jw) ^ __double2hiint(jp);
+                if (sj < 0 || (__double2hiint(jw) & 0x7fffffff) > 0x7ff00000) continue;
+                const R cf = lam * jw;
+#pragma unroll
+                for (int q = 0; q < NC; ++q)
+                    if (q >= q0) Fd[q] = fma(rc[q], cf, Fd[q]);
+                continue;
+            } else {
             R Wm, Wp, jp;
             if constexpr (std::is_same<R, float>::value && WK == 0) {
                 // binary32 WENO-MR: the node pairs (0,5), (1,4), (2,3) of the two stencils in paired lanes
@@ -623,6 +853,7 @@ __device__ __forceinline__ void iface_flux(const Inst& I, const R* nb, int NN, i
 #pragma unroll
                 for (int q = 0; q < NC; ++q) Fd[q] += rc[q] * cf;
             }
+            }
         }
 #pragma unroll
         for (int q = 0; q < NC; ++q) fl[q * NI + f] = fl[q * NI + f] - R(0.5) * Fd[q];
@@ -650,10 +881,14 @@ __device__ __forceinline__ void node_div(const Inst& I, const R* fl, int NI, con
     R rdx;
     if constexpr (std::is_same<R, float>::value) rdx = I.f_inv_dxi[k];
     else rdx = inv_dx;
-    r[NC] = -(gt[fr] - gt[fL]) * inv_dx;
+    r[NC] = __dmul_rn(-(gt[fr] - gt[fL]), inv_dx);
 #pragma unroll
-    for (int q = 0; q < NC; ++q) r[q] = to_d(-(fl[q * NI + fr] - fl[q * NI + fL]) * rdx);
-    r[NC - 1] += I.pinf_tot * r[NC];
+    for (int q = 0; q < NC; ++q) {
+        // (a rounded product: the sums over the directions start from it)
+        if constexpr (std::is_same<R, double>::value) r[q] = __dmul_rn(-(fl[q * NI + fr] - fl[q * NI + fL]), rdx);
+        else r[q] = to_d(-(fl[q * NI + fr] - fl[q * NI + fL]) * rdx);
+    }
+    r[NC - 1] = fma(I.pinf_tot, r[NC], r[NC - 1]);
 }
 
 }  // namespace es

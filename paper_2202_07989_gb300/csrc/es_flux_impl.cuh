@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(FLUX_TPB, (sizeof(R) == 4 ? (D == 3 ? 4 : 3) :
                     const long long id = staged ? 0 : lin(I, src[0], src[1], src[2]);
                     const R inv = Ar<R>::rcp(to_r<R>(staged ? stg[NC * NN + node] : P.J[id]));
 #pragma unroll
-                    for (int q = 0; q < NC; ++q) U[q] = to_r<R>(staged ? stg[q * NN + node] : P.JU[q * ncell + id]) * inv;
+                    for (int q = 0; q < NC; ++q) U[q] = mulr(to_r<R>(staged ? stg[q * NN + node] : P.JU[q * ncell + id]), inv);
                     if (tmap == 1) U[NS + k] = -U[NS + k];
                 }
             }
