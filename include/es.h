@@ -179,8 +179,11 @@ es_status es_autotune(es_ctx* ctx, const double* JU, const double* J, const doub
 
 /* The flux launch configuration per direction k = 0..2 (zeros for directions
  * the problem lacks): shape index, S, WT, persistent grid size (CTAs) and the
- * time per launch the last es_autotune measured (0 if none).  Each argument
- * points to 3 values (HOST). */
+ * time per launch the last es_autotune measured (0 if none).  A 3D context that
+ * nobody tuned picks its tiles by its grid; in the FP64 form, and in es_autotune
+ * there, they may have an extent of their own: S and WT are then that extent and
+ * the shape index the one it replaces.
+ * Each argument points to 3 values (HOST). */
 es_status es_get_tuning(const es_ctx* ctx, int* shape, int* S, int* WT, int* grid, float* ms);
 
 /* Fix the flux launch of direction k to tile shape `shape` (0..5) and `grid`

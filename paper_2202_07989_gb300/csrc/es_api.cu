@@ -5,6 +5,7 @@
 #include "../../include/es.h"
 #include "es_mesh.cuh"
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -29,8 +30,11 @@ struct es_ctx {
     int2* w_xe = nullptr;   int n_xe = 0;      // 3D FP64 form: nodes within 9 ghost layers
     int2* w_cell = nullptr; int n_cell = 0;
     int2* w_col = nullptr;  int n_col = 0;     // 3D: column chunks of the kernels marching along i3
-    int2* w_flux[3][NSHAPE] = {};          // flux work list per direction and tile shape
-    int n_flux[3][NSHAPE] = {};
+    // flux work list per direction and tile shape; the last one (3D) is the extent fitted to the grid
+    int2* w_flux[3][NSHAPE + 1] = {};
+    int n_flux[3][NSHAPE + 1] = {};
+    int fit_S[3] = { 0, 0, 0 }, fit_WT[3] = { 0, 0, 0 };
+    bool flux_fit[3] = { false, false, false };    // the launches use the fitted extent
     int2* w_fused[NFSHAPE_ALL] = {};           // fused 2D stage work list per fused tile shape
     int n_fused[NFSHAPE_ALL] = {};
     int2* w_jf[NJF_SHAPE_ALL] = {};            // mixed 2D: fused mesh-step tiles per shape (JF_SHAPES)
@@ -264,10 +268,23 @@ void prepare_all(int weno)
     }
 }
 
+int gcd_(int a, int b) { return b == 0 ? a : gcd_(b, a % b); }
+
+// The largest grid up to `grid` CTAs that shares no factor with the segments per line (ns): tiles
+// are numbered segment by segment, so with a common factor the same CTAs would get every line's
+// last, partial segment and the others only full ones (direction 1 of 63^3 in the FP64 form, 62 x 4
+// tiles: 1737 us with 152 CTAs, 1126 us with the partial tiles spread)
+int spread_grid(int grid, int ns)
+{
+    while (grid > 1 && gcd_(grid, ns) != 1) --grid;
+    return grid;
+}
+
 // one flux launch in the given tile shape and grid
 void flux_launch(es_ctx* c, const FluxLaunch& L, int shape, int grid, cudaStream_t st)
 {
     if (grid > L.nwork) grid = L.nwork;
+    else if (c->d == 3 && c->n_inst == 1) grid = spread_grid(grid, (c->hI[0].n[L.k] + L.S - 1) / L.S);
     if (grid <= 0) return;
 #define FD(d, n)                                                                                      \
     do {                                                                                              \
@@ -332,14 +349,16 @@ void pick_fused(es_ctx* c)
     }
 }
 
-// flux tiles of instance I along direction k in tile shape `shape`
-long long flux_tiles(const Inst& I, int k, int shape)
+// flux tiles of S nodes along the line x WT lines of instance I along direction k
+long long flux_tiles(const Inst& I, int k, int S, int WT)
 {
-    const int S = SHAPE_S[shape], WT = SHAPE_WT[shape];
     const int adim = k == 0 ? 1 : 0, bdim = k == 2 ? 1 : 2;
     const long long nb = bdim < I.d ? I.n[bdim] : 1;
     return (long long)((I.n[k] + S - 1) / S) * ((I.n[adim] + WT - 1) / WT) * nb;
 }
+
+int shape_S(const es_ctx* c, int k, int sh) { return sh < NSHAPE ? SHAPE_S[sh] : c->fit_S[k]; }
+int shape_WT(const es_ctx* c, int k, int sh) { return sh < NSHAPE ? SHAPE_WT[sh] : c->fit_WT[k]; }
 
 int flux_occ(es_ctx* c, int shape)
 {
@@ -353,6 +372,79 @@ int flux_occ(es_ctx* c, int shape)
     if (c->d == 3 && c->N == 1) FO(3, 1);
     FO(3, 2);
 #undef FO
+}
+
+// The time of a 3D flux tile of s nodes along the line x w lines, in arbitrary units.
+// Mixed form: a fixed part (a tile's phases wait on one another and on their loads), one unit per
+// round of nodes over the 256 threads and 0.4 per warp of pairs; loads across the contiguous
+// direction favour more lines (fitted to six shapes on 128^3, 100^3, 128x64x64 and 400x80x80 grids:
+// the order of the shapes and their ratios within 8%).  FP64 form: the FP64 pipe of each of the
+// SM's four partitions takes 64 cycles a warp instruction, so a phase takes its instructions per
+// thread times the warps of one partition (a single warp there waits for its own results).
+double tile_cost_3d(bool mixed, int k, int s, int w)
+{
+    auto rounds = [](int items, int per) { return (items + per - 1) / per; };
+    const int nodes = (s + 6) * w, pairs = (3 * s + 6) * w, ifaces = (s + 1) * w;
+    if (!mixed) {
+        auto r = [&](int items) { return items <= 32 ? 2.1 : (items <= 128 ? 1.6 : (double)rounds(items, 128)); };
+        return 200.0 * r(nodes) + 85.0 * r(pairs) + 1050.0 * r(ifaces);
+    }
+    const double t = 4.0 + rounds(nodes, FLUX_TPB) + 0.4 * rounds(pairs, 32);
+    return k == 0 || w >= 8 ? t : t * (w >= 4 ? 1.05 : 1.37);
+}
+
+// time of all tiles of S x WT along direction k, dealt over the grid's CTAs
+double tiles_cost_3d(const es_ctx* c, int k, int S, int WT, int slots)
+{
+    const int grid = c->n_inst == 1 ? spread_grid(slots, (c->hI[0].n[k] + S - 1) / S) : slots;
+    std::vector<double> load(grid, 0.0);
+    double sum = 0.0, top = 0.0;
+    long long t = 0;
+    for (const Inst& I : c->hI) {
+        const int na = I.n[k == 0 ? 1 : 0], nb = I.n[k == 2 ? 1 : 2];
+        for (int b = 0; b < nb; ++b)
+            for (int a = 0; a < na; a += WT)
+                for (int q = 0; q < I.n[k]; q += S, ++t) {
+                    const double w = tile_cost_3d(c->mixed, k, std::min(S, I.n[k] - q), std::min(WT, na - a));
+                    sum += w;
+                    double& l = load[t % grid];
+                    l += w;
+                    top = std::max(top, l);
+                }
+    }
+    return t > 8LL * grid ? sum / grid : top;     // many waves: the mean
+}
+
+// The 3D flux tile of direction k for a context that nobody tuned.  Mixed form: the shape of the
+// table whose tiles finish first (128^3: 26 x 8 in every direction, 1017 us for the three launches
+// of a stage where the fixed 62 x 4 and 30 x 8 took 1134).  FP64 form: over all line counts, the
+// longest segment that leaves one interface per thread and the one that divides the lines evenly
+// (63^3: 63 x 4, 2563 us for the three launches; the fixed shapes 3770, the table's best 2650).
+void pick_tiles_3d(es_ctx* c, int k, int slots)
+{
+    double best = 0.0;
+    if (c->mixed) {
+        for (int sh = 0; sh < NSHAPE; ++sh) {
+            const double cost = tiles_cost_3d(c, k, SHAPE_S[sh], SHAPE_WT[sh], slots);
+            if (sh == 0 || cost < best) {
+                best = cost;
+                c->flux_shape[k] = sh;
+            }
+        }
+        return;
+    }
+    for (int WT = 1; WT <= FLUX_WT_MAX; ++WT) {
+        const int smax = FLUX_TPB / WT - 1, n0 = c->hI[0].n[k], parts = (n0 + smax - 1) / smax;
+        for (int S : { smax, (n0 + parts - 1) / parts }) {
+            const double cost = tiles_cost_3d(c, k, S, WT, slots);
+            if (c->fit_S[k] == 0 || cost < best) {
+                best = cost;
+                c->fit_S[k] = S;
+                c->fit_WT[k] = WT;
+            }
+        }
+    }
+    c->flux_fit[k] = true;
 }
 
 // planes per chunk of the 3D kernels that march along i3: chunks enough for about four
@@ -480,7 +572,9 @@ void launch_residual(es_ctx* c, const StagePtrs& P, const StagePtrs* tab, bool r
         L.insts = c->dI;
         L.single = P;
         L.ptrs = tab;
-        const int sh = c->flux_shape[k];
+        const int sh = c->flux_fit[k] ? NSHAPE : c->flux_shape[k];
+        L.S = shape_S(c, k, sh);
+        L.WT = shape_WT(c, k, sh);
         L.work = c->w_flux[k][sh];
         L.nwork = c->n_flux[k][sh];
         L.k = k;
@@ -775,7 +869,8 @@ es_status es_create_batch(const es_config* cfgs, int n_inst, es_ctx** out)
     if (c->d == 3 && !c->mixed) c->w_xe = build_work(c, [](const Inst& I) { return (long long)node_tiles(I, 9); }, c->n_xe);
     for (int k = 0; k < c->d; ++k)
         for (int sh = 0; sh < NSHAPE; ++sh) {
-            c->w_flux[k][sh] = build_work(c, [k, sh](const Inst& I) { return flux_tiles(I, k, sh); }, c->n_flux[k][sh]);
+            c->w_flux[k][sh] = build_work(c, [k, sh](const Inst& I) { return flux_tiles(I, k, SHAPE_S[sh], SHAPE_WT[sh]); },
+                                          c->n_flux[k][sh]);
             ok = ok && c->w_flux[k][sh];
         }
     if (c->d == 2)
@@ -803,7 +898,18 @@ es_status es_create_batch(const es_config* cfgs, int n_inst, es_ctx** out)
     else if (c->d == 3 && c->N == 1) prepare_all<3, 1>(c->weno);
     else prepare_all<3, 2>(c->weno);
     prepare_mesh();
-    for (int k = 0; k < c->d; ++k) c->flux_grid[k] = c->sms * flux_occ(c, c->flux_shape[k]);
+    for (int k = 0; k < c->d; ++k) {
+        c->flux_grid[k] = c->sms * flux_occ(c, c->flux_shape[k]);
+        if (c->d != 3) continue;
+        pick_tiles_3d(c, k, c->flux_grid[k]);
+        if (c->mixed) {
+            c->flux_grid[k] = c->sms * flux_occ(c, c->flux_shape[k]);
+            continue;
+        }
+        const int S = c->fit_S[k], WT = c->fit_WT[k];
+        c->w_flux[k][NSHAPE] = build_work(c, [k, S, WT](const Inst& I) { return flux_tiles(I, k, S, WT); }, c->n_flux[k][NSHAPE]);
+        ok = ok && c->w_flux[k][NSHAPE];
+    }
     // 2D contexts start with the fused stage launch in fused shape 0 (es_autotune may change it)
     if (c->d == 2) {
         c->fused_shape = 0;
@@ -1123,13 +1229,16 @@ es_status es_autotune(es_ctx* c, const double* JU, const double* J, const double
     cudaEventCreate(&e1);
     for (int k = 0; k < c->d; ++k) {
         float best = 3.0e38f;
-        for (int sh = 0; sh < NSHAPE; ++sh) {
+        c->flux_fit[k] = false;
+        for (int sh = 0; sh < NSHAPE + (c->fit_S[k] > 0); ++sh) {
             const int occ = flux_occ(c, sh);
             for (int o = occ; o >= 1 && o >= occ - 1; --o) {
                 FluxLaunch L;
                 L.insts = c->dI;
                 L.single = P;
                 L.ptrs = tab;
+                L.S = shape_S(c, k, sh);
+                L.WT = shape_WT(c, k, sh);
                 L.work = c->w_flux[k][sh];
                 L.nwork = c->n_flux[k][sh];
                 L.k = k;
@@ -1150,7 +1259,8 @@ es_status es_autotune(es_ctx* c, const double* JU, const double* J, const double
                 ms /= (float)reps;
                 if (ms < best) {
                     best = ms;
-                    c->flux_shape[k] = sh;
+                    if (sh < NSHAPE) c->flux_shape[k] = sh;
+                    else c->flux_fit[k] = true;
                     c->flux_grid[k] = grid;
                 }
             }
@@ -1273,8 +1383,9 @@ es_status es_get_tuning(const es_ctx* c, int* shape, int* S, int* WT, int* grid,
     for (int k = 0; k < 3; ++k) {
         const bool on = k < c->d;
         shape[k] = on ? c->flux_shape[k] : 0;
-        S[k] = on ? SHAPE_S[c->flux_shape[k]] : 0;
-        WT[k] = on ? SHAPE_WT[c->flux_shape[k]] : 0;
+        const int sh = on && c->flux_fit[k] ? NSHAPE : c->flux_shape[k];
+        S[k] = on ? shape_S(c, k, sh) : 0;
+        WT[k] = on ? shape_WT(c, k, sh) : 0;
         grid[k] = on ? c->flux_grid[k] : 0;
         ms[k] = on ? c->flux_ms[k] : 0.f;
     }
@@ -1287,6 +1398,7 @@ es_status es_set_tuning(es_ctx* c, int k, int shape, int grid)
     if (k < 0 || k >= c->d || shape < 0 || shape >= NSHAPE || grid < 0)
         return fail(c, ES_ERR_ARG, "es_set_tuning: direction, shape or grid out of range");
     c->flux_shape[k] = shape;
+    c->flux_fit[k] = false;
     c->flux_grid[k] = grid > 0 ? grid : c->sms * flux_occ(c, shape);
     c->flux_ms[k] = 0.f;
     drop_run_graph(c);

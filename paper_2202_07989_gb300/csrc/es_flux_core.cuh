@@ -35,48 +35,64 @@ struct Ar<double> {
     static __device__ __forceinline__ double lg(double x) { return log(x); }
     static __device__ __forceinline__ double sq(double x) { return sqrt(x); }
     static __device__ __forceinline__ double ab(double x) { return fabs(x); }
-    // |dd| < s / 128, on the high words: no FP64 comparison (it would issue on the FP64 pipe).
-    // Series and quotient agree to round-off around this threshold, so its last bits are free.
-    static __device__ __forceinline__ bool small_jump(double dd, double s)
+    // |dd| < s / 2^e, on the high words: no FP64 comparison (it would issue on the FP64 pipe).
+    // Series and quotient agree to round-off around the thresholds, so their last bits are free.
+    static __device__ __forceinline__ bool jump_below(double dd, double s, int e)
     {
-        return (__double2hiint(dd) & 0x7fffffff) < __double2hiint(s) - (7 << 20);
+        return (__double2hiint(dd) & 0x7fffffff) < __double2hiint(s) - (e << 20);
+    }
+    // f / artanh(f) and artanh(f) / f in u = f^2: four terms for |f| < 2^-7, nine for |f| < 2^-3 (a
+    // logarithm takes more FP64 instructions than the five terms, and a warp pays for it when any
+    // of its lanes needs one)
+    static __device__ __forceinline__ double series_ln(double u, bool tiny)
+    {
+        double p = -44.0 / 945.0;
+        if (!tiny)
+            p = fma(u, fma(u, fma(u, fma(u, fma(u, -5472607916.0 / 488462349375.0, -25865068.0 / 1915538625.0),
+                                         -10719068.0 / 638512875.0), -10196.0 / 467775.0), -428.0 / 14175.0), p);
+        return fma(u, fma(u, fma(u, p, -4.0 / 45.0), -1.0 / 3.0), 1.0);
+    }
+    static __device__ __forceinline__ double series_inv(double u, bool tiny)
+    {
+        double p = 1.0 / 7.0;
+        if (!tiny) p = fma(u, fma(u, fma(u, fma(u, fma(u, 1.0 / 17.0, 1.0 / 15.0), 1.0 / 13.0), 1.0 / 11.0), 1.0 / 9.0), p);
+        return fma(u, fma(u, fma(u, p, 1.0 / 5.0), 1.0 / 3.0), 1.0);
     }
     // {a}^ln: [[a]]/[[ln a]], Ismail-Roe series at small jumps; is = 1/(a + b)
     static __device__ __forceinline__ double lmean_is(double a, double b, double is, double la, double lb)
     {
         const double s = a + b, dd = b - a;
-        if (small_jump(dd, s)) {
-            const double f = dd * is, u = f * f;
-            return __dmul_rn(0.5 * s, fma(-u, fma(u, fma(u, 44.0 / 945.0, 4.0 / 45.0), 1.0 / 3.0), 1.0));
+        if (jump_below(dd, s, 3)) {
+            const double f = dd * is;
+            return __dmul_rn(0.5 * s, series_ln(f * f, jump_below(dd, s, 7)));
         }
         return dd / (lb - la);
     }
     // 1/{a}^ln
     static __device__ __forceinline__ double inv_lmean(double a, double b, double la, double lb, double is)
     {
-        const double dd = b - a;
-        if (small_jump(dd, a + b)) {
-            const double f = dd * is, u = f * f;
-            return __dmul_rn(2.0 * is, fma(u, fma(u, fma(u, 1.0 / 7.0, 1.0 / 5.0), 1.0 / 3.0), 1.0));
+        const double s = a + b, dd = b - a;
+        if (jump_below(dd, s, 3)) {
+            const double f = dd * is;
+            return __dmul_rn(2.0 * is, series_inv(f * f, jump_below(dd, s, 7)));
         }
         return (lb - la) / dd;
     }
     // the same with the logarithms formed only in their branch
     static __device__ __forceinline__ double lmean_is(double a, double b, double is)
     {
-        if (small_jump(b - a, a + b)) return lmean_is(a, b, is, 0.0, 0.0);
-        return (b - a) / (lg(b) - lg(a));
+        if (jump_below(b - a, a + b, 3)) return lmean_is(a, b, is, 0.0, 0.0);
+        return (b - a) / __dsub_rn(lg(b), lg(a));
     }
     static __device__ __forceinline__ double lmean(double a, double b)
     {
-        if (small_jump(b - a, a + b)) return lmean_is(a, b, 1.0 / (a + b), 0.0, 0.0);
-        return (b - a) / (lg(b) - lg(a));
+        if (jump_below(b - a, a + b, 3)) return lmean_is(a, b, 1.0 / (a + b), 0.0, 0.0);
+        return (b - a) / __dsub_rn(lg(b), lg(a));
     }
     static __device__ __forceinline__ double inv_lmean(double a, double b, double is)
     {
-        const double dd = b - a;
-        if (small_jump(dd, a + b)) return inv_lmean(a, b, 0.0, 0.0, is);
-        return (lg(b) - lg(a)) / dd;
+        if (jump_below(b - a, a + b, 3)) return inv_lmean(a, b, 0.0, 0.0, is);
+        return __dsub_rn(lg(b), lg(a)) / (b - a);
     }
 };
 
@@ -135,6 +151,9 @@ __device__ __forceinline__ double dot2(double a, double b, double c, double d) {
 __device__ __forceinline__ float dot2(float a, float b, float c, float d) { return a * b + c * d; }
 __device__ __forceinline__ double mad(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float mad(float a, float b, float c) { return a * b + c; }
+// term i of the sum of products s += a b (s = 0 before term 0)
+__device__ __forceinline__ double acc_prod(int i, double a, double b, double s) { return i == 0 ? __dmul_rn(a, b) : fma(a, b, s); }
+__device__ __forceinline__ float acc_prod(int, float a, float b, float s) { return s + a * b; }
 __device__ __forceinline__ double mulr(double a, double b) { return __dmul_rn(a, b); }     // never fused
 __device__ __forceinline__ float mulr(float a, float b) { return a * b; }
 
@@ -342,7 +361,7 @@ __device__ __forceinline__ R vnorm(const R* nb, int NN)
 {
     R vn = R(0);
 #pragma unroll
-    for (int q = 0; q < NC; ++q) vn += nb[(VV + q) * NN] * nb[(VV + q) * NN];
+    for (int q = 0; q < NC; ++q) vn = acc_prod(q, nb[(VV + q) * NN], nb[(VV + q) * NN], vn);
     return Ar<R>::sq(vn);
 }
 
@@ -359,7 +378,7 @@ __device__ __forceinline__ void node_fields(const Inst& I, const R* U, R* nr, in
     R irho = Ar<R>::rcp(rho);
     R v[D], v2 = R(0);
 #pragma unroll
-    for (int m = 0; m < D; ++m) { v[m] = U[NS + m] * irho; v2 += v[m] * v[m]; }
+    for (int m = 0; m < D; ++m) { v[m] = U[NS + m] * irho; v2 = acc_prod(m, v[m], v[m], v2); }
     R cvr, rhoe_p;
     if constexpr (std::is_same<R, double>::value) {
         cvr = NS == 2 ? dot2(I.cv[0], U[0], I.cv[1], U[1]) : I.cv[0] * U[0];
@@ -420,7 +439,7 @@ __device__ __forceinline__ void node_fields(const Inst& I, const R* U, R* nr, in
     Vn[NS + D] = -beta;
     R vn = R(0);
 #pragma unroll
-    for (int q = 0; q < NC; ++q) { nr[(Y::VV + q) * NN + node] = Vn[q]; vn += Vn[q] * Vn[q]; }
+    for (int q = 0; q < NC; ++q) { nr[(Y::VV + q) * NN + node] = Vn[q]; vn = acc_prod(q, Vn[q], Vn[q], vn); }
     if constexpr (!Y::COMPACT) nr[Y::VN * NN + node] = Ar<R>::sq(vn);
 }
 
@@ -587,7 +606,7 @@ __device__ __forceinline__ void iface_flux(const Inst& I, const R* nb, int NN, i
             const int fj = mr + 1 + j;
             Gx[j] = mad(Cst<R>::gcw(I, 2), NR(fj, 0) + NR(fj, 5), dot2(Cst<R>::gcw(I, 0), NR(fj, 2) + NR(fj, 3),
                                                                        Cst<R>::gcw(I, 1), NR(fj, 1) + NR(fj, 4)));
-            L2 += Gx[j] * Gx[j];
+            L2 = acc_prod(j, Gx[j], Gx[j], L2);
         }
         R Ln = Ar<R>::sq(L2), iL = Ar<R>::rcp(Ln);
         R n[D];
@@ -615,12 +634,12 @@ __device__ __forceinline__ void iface_flux(const Inst& I, const R* nb, int NN, i
         const R Tb = cm[NS * NI + f];       // T-bar = 1 / {beta}^ln
         R vb[D], vh[D], vv = R(0);
 #pragma unroll
-        for (int j = 0; j < D; ++j) { vb[j] = R(0.5) * (NR(Y::V + j, 2) + NR(Y::V + j, 3)); vv += vb[j] * vb[j]; }
+        for (int j = 0; j < D; ++j) { vb[j] = R(0.5) * (NR(Y::V + j, 2) + NR(Y::V + j, 3)); vv = acc_prod(j, vb[j], vb[j], vv); }
 #pragma unroll
         for (int m = 0; m < D; ++m) {
             R s_ = R(0);
 #pragma unroll
-            for (int j = 0; j < D; ++j) s_ += T[m][j] * vb[j];
+            for (int j = 0; j < D; ++j) s_ = acc_prod(j, T[m][j], vb[j], s_);
             vh[m] = s_;
         }
         R cb, H, sa, se = R(0), ssh, Y1 = R(1), Y2 = R(0), D11 = R(0), D12 = R(0), D21 = R(0), D22 = R(0), e1 = R(0), e2 = R(0);
@@ -672,12 +691,12 @@ __device__ __forceinline__ void iface_flux(const Inst& I, const R* nb, int NN, i
                 const double pre = sqrt(rg), psy = sqrt(rg * (Y1 * Y2) * Gb), psg = pre * (gm * ig);
                 sa = pre * 0.70710678118654752440;
                 ssh = sqrt(rb * Tb);
-                D11 = -psy * I.sq21;
-                D21 = psy * I.sq12;
-                D12 = psg * Y1;
-                D22 = psg * Y2;
-                e1 = fma(-(I.cv[0] + I.Rs[0] - Gb * I.cv[0]) * Tb, igm, 0.5 * vv);
-                e2 = fma(-(I.cv[1] + I.Rs[1] - Gb * I.cv[1]) * Tb, igm, 0.5 * vv);
+                D11 = -__dmul_rn(psy, I.sq21);
+                D21 = __dmul_rn(psy, I.sq12);
+                D12 = __dmul_rn(psg, Y1);
+                D22 = __dmul_rn(psg, Y2);
+                e1 = fma(-fma(-Gb, I.cv[0], I.cv[0] + I.Rs[0]) * Tb, igm, 0.5 * vv);
+                e2 = fma(-fma(-Gb, I.cv[1], I.cv[1] + I.Rs[1]) * Tb, igm, 0.5 * vv);
             } else {
             const R pre = Ar<R>::sq(rb * Ar<R>::rcp(Gb * Rb));
             sa = pre * R(0.70710678118654752440);
@@ -768,7 +787,7 @@ __device__ __forceinline__ void iface_flux(const Inst& I, const R* nb, int NN, i
             for (int j = 0; j < D; ++j) {
                 R s_ = R(0);
 #pragma unroll
-                for (int m = 0; m < D; ++m) s_ += T[m][j] * rc[NS + m];
+                for (int m = 0; m < D; ++m) s_ = acc_prod(m, T[m][j], rc[NS + m], s_);
                 ru[j] = s_;
             }
 #pragma unroll

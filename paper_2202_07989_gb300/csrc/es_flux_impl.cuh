@@ -15,8 +15,16 @@ template <int S, int WT>
 struct Tile {
     static constexpr int NN = (S + 6) * WT;   // staged nodes (3 halo nodes per side)
     static constexpr int NI = (S + 1) * WT;   // interfaces
-    static constexpr int NPL = 3 * S + 6;     // distinct node pairs (j, j+m), m = 1..3, per line
-    static constexpr int NP = NPL * WT;
+    static constexpr int NP = (3 * S + 6) * WT;   // distinct node pairs (j, j+m), m = 1..3
+};
+// The 3D FP64 tiles (S = WT = 0 here) get their extent with the launch: any S and WT <=
+// FLUX_WT_MAX with (S + 1) WT <= 256, in arrays of the capacity of the widest.  The mixed form
+// keeps its extents at compile time: with run-time ones its 3D launches took 3-5% longer
+template <>
+struct Tile<0, 0> {
+    static constexpr int NN = FLUX_TPB + 5 * FLUX_WT_MAX;
+    static constexpr int NI = FLUX_TPB;
+    static constexpr int NP = 3 * FLUX_TPB + 3 * FLUX_WT_MAX;
 };
 
 // rows of the staging buffer: JU (n_c), J and the metric row of direction k (d + 1); a 2D
@@ -93,6 +101,10 @@ __device__ __forceinline__ void flux_stage(const FluxLaunch& L, int k, int wi, d
     cp_async_commit();
 }
 
+// t / n for 0 <= t < 4096 and 1 <= n <= 512, given r = 1/n in binary32: (t + 1/2) r is off the exact
+// quotient by less than 4096 * 2^-23 < 1 / (2n), so its integer part is t / n
+__device__ __forceinline__ int div_small(int t, float r) { return (int)(((float)t + 0.5f) * r); }
+
 // Phases of one tile: (1) node states, entropy variables and metrics into shared memory;
 // (2) every distinct two-point flux F(U_j, U_{j+m}) (m = 1, 2, 3) of the tile, once; (3)
 // per interface the 2w-order EC flux as sum_m alpha_m sum_s of the stored pairs, the GCL
@@ -100,13 +112,15 @@ __device__ __forceinline__ void flux_stage(const FluxLaunch& L, int k, int wi, d
 // FP32 tiles: 3 CTAs per SM in 2D (<= 85 registers), 4 in 3D (<= 64 registers: the compact 3D
 // node layout and no staging buffer leave room for 4, measured 3-10% faster than 3 with the
 // staging buffer, spills included); FP64 tiles: 1 (FP64-pipe bound)
-template <int D, int NS, typename R, int S, int WT, int WK>
+template <int D, int NS, typename R, int S_, int WT_, int WK>
 __global__ void __launch_bounds__(FLUX_TPB, (sizeof(R) == 4 ? (D == 3 ? 4 : 3) : 1)) flux_kernel(FluxLaunch L)
 {
     pdl_entry();
     using Y = Lay<D, NS>;
-    using TL = Tile<S, WT>;
-    constexpr int NC = Y::NC, NN = TL::NN, NI = TL::NI, NF = Y::NF, NPL = TL::NPL, NP = TL::NP;
+    using TL = Tile<S_, WT_>;
+    constexpr int NC = Y::NC, NN = TL::NN, NI = TL::NI, NF = Y::NF, NP = TL::NP;
+    static_assert(NP < 4096 && 3 * S_ + 6 <= 512, "div_small");
+    const int S = S_ > 0 ? S_ : L.S, WT = S_ > 0 ? WT_ : L.WT, NPL = 3 * S + 6;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double* gt = reinterpret_cast<double*>(smem_raw);           // [NI] GCL flux of J xi_k/t
     double* mt64 = gt + NI;                                      // [NN] J xi_k/t at the nodes
@@ -114,7 +128,7 @@ __global__ void __launch_bounds__(FLUX_TPB, (sizeof(R) == 4 ? (D == 3 ? 4 : 3) :
     R* pf = nr + NF * NN;                                        // [NC][NP] pair fluxes
     R* cm = pf + NC * NP;                                        // [NS + 1][NI] centre-pair means
     R* fl = cm + (NS + 1) * NI;                                  // [NC][NI] interface fluxes
-    double* stg = reinterpret_cast<double*>(smem_raw + stage_offset<D, NS, R, S, WT>());   // [NC + D + 2][NN]
+    double* stg = reinterpret_cast<double*>(smem_raw + stage_offset<D, NS, R, S_, WT_>());   // [NC + D + 2][NN]
     const int k = L.k;
     const int adim = k == 0 ? 1 : 0, bdim = k == 2 ? 1 : 2;
 
@@ -123,7 +137,8 @@ __global__ void __launch_bounds__(FLUX_TPB, (sizeof(R) == 4 ? (D == 3 ? 4 : 3) :
     // buffer, so their loads overlap phases 2-4.  With one tile per CTA there is nothing to
     // overlap, and phase 1 loads directly.
     const bool staged = stages_inputs<D, NS>() && L.nwork > (int)gridDim.x;
-    if (staged && blockIdx.x < L.nwork) flux_stage<D, NS, S, WT>(L, k, blockIdx.x, stg);
+    if constexpr (stages_inputs<D, NS>())
+        if (staged && blockIdx.x < L.nwork) flux_stage<D, NS, S_, WT_>(L, k, blockIdx.x, stg);
     for (int wi = blockIdx.x; wi < L.nwork; wi += gridDim.x) {
         const int2 it = L.work[wi];
         const Inst& I = L.insts[it.x];
@@ -133,6 +148,11 @@ __global__ void __launch_bounds__(FLUX_TPB, (sizeof(R) == 4 ? (D == 3 ? 4 : 3) :
         const int ts = it.y % ns, ta = (it.y / ns) % nat, tb = it.y / (ns * nat);
         const int s0 = ts * S, a0 = ta * WT;
         const long long ncell = I.ncell;
+        // the tile's own extent: its items are numbered over the nodes it has, so that the last,
+        // partial tile of a line or of the plane costs what it holds
+        const int sE = min(S, nk - s0), wE = min(WT, na - a0);
+        const float rN = 1.0f / (float)(sE + 6), rW = 1.0f / (float)wE, rP = 1.0f / (float)(3 * sE + 6),
+                    rI = 1.0f / (float)(sE + 1), rS = 1.0f / (float)sE;
         // 2D stage metrics M + s Md with s = mcoef dt (the stage mesh is x^n + s xdot)
         const double sM = (D == 2 && L.mcoef != 0.0) ? L.mcoef * *P.dt : 0.0;
 
@@ -141,17 +161,12 @@ __global__ void __launch_bounds__(FLUX_TPB, (sizeof(R) == 4 ? (D == 3 ? 4 : 3) :
             cp_async_wait_all();
             __syncthreads();
         }
-        for (int t = threadIdx.x; t < NN; t += blockDim.x) {
+        for (int t = threadIdx.x; t < (sE + 6) * wE; t += blockDim.x) {
             int s, w;
-            if (k == 0) { s = t % (S + 6); w = t / (S + 6); }
-            else { w = t % WT; s = t / WT; }
+            if (k == 0) { w = div_small(t, rN); s = t - w * (sE + 6); }
+            else { s = div_small(t, rW); w = t - s * wE; }
             const int node = w * (S + 6) + s;
             const int g = s0 - 3 + s, a = a0 + w;
-            if (a >= na || g > nk + 2) {
-                for (int f = 0; f < NF; ++f) nr[f * NN + node] = R(1);
-                mt64[node] = 0.0;
-                continue;
-            }
             int idx[3] = { 0, 0, 0 };
             idx[k] = g;
             idx[adim] = a;
@@ -195,26 +210,26 @@ __global__ void __launch_bounds__(FLUX_TPB, (sizeof(R) == 4 ? (D == 3 ? 4 : 3) :
             }
         }
         __syncthreads();
-        if (staged && wi + (int)gridDim.x < L.nwork) flux_stage<D, NS, S, WT>(L, k, wi + (int)gridDim.x, stg);
+        if constexpr (stages_inputs<D, NS>())
+            if (staged && wi + (int)gridDim.x < L.nwork) flux_stage<D, NS, S_, WT_>(L, k, wi + (int)gridDim.x, stg);
 
         // ---------------- phase 2: distinct two-point EC fluxes ----------------
-        for (int t = threadIdx.x; t < NP; t += blockDim.x) {
-            const int w = t / NPL, r_ = t % NPL;
-            int m, Ln;
-            if (r_ < S + 1) { m = 1; Ln = r_ + 2; }
-            else if (r_ < 2 * S + 3) { m = 2; Ln = r_ - (S + 1) + 1; }
-            else { m = 3; Ln = r_ - (2 * S + 3); }
-            if (a0 + w >= na || s0 - 3 + Ln + m > nk + 2) continue;
+        for (int t = threadIdx.x; t < (3 * sE + 6) * wE; t += blockDim.x) {
+            const int w = div_small(t, rP), r_ = t - w * (3 * sE + 6);
+            // the pair's kind m, its left node Ln and its place among the line's NPL pairs
+            int m, Ln, pl;
+            if (r_ < sE + 1) { m = 1; Ln = r_ + 2; pl = r_; }
+            else if (r_ < 2 * sE + 3) { m = 2; Ln = r_ - (sE + 1) + 1; pl = r_ - sE + S; }
+            else { m = 3; Ln = r_ - (2 * sE + 3); pl = r_ - 2 * sE + 2 * S; }
             const int l = w * (S + 6) + Ln;
-            pair_flux<D, NS, R>(I, nr, NN, Y::MR, l, l + m, pf, NP, t, cm, NI, m == 1 ? w * (S + 1) + (Ln - 2) : -1);
+            pair_flux<D, NS, R>(I, nr, NN, Y::MR, l, l + m, pf, NP, w * NPL + pl, cm, NI, m == 1 ? w * (S + 1) + (Ln - 2) : -1);
         }
         __syncthreads();
 
         // ---------------- phase 3: interface fluxes ----------------
-        for (int f = threadIdx.x; f < NI; f += blockDim.x) {
-            const int s = f % (S + 1), w = f / (S + 1);
-            const int gi = s0 - 1 + s;     // interface gi + 1/2
-            if (a0 + w >= na || gi > nk - 1) continue;
+        for (int t = threadIdx.x; t < (sE + 1) * wE; t += blockDim.x) {
+            const int w = div_small(t, rI), s = t - w * (sE + 1);     // interface s0 - 1 + s + 1/2
+            const int f = w * (S + 1) + s;
             const int base = w * (S + 6) + s;   // node gi - 2
             const int p1 = w * NPL + s, p2 = w * NPL + (S + 1) + s, p3 = w * NPL + (2 * S + 3) + s;
             iface_flux<D, NS, R, WK>(I, nr + base, NN, 1, Y::MR, mt64 + base, 1, pf, NP, p1, p2, p3, 1, cm, NI, f, fl, gt);
@@ -223,12 +238,11 @@ __global__ void __launch_bounds__(FLUX_TPB, (sizeof(R) == 4 ? (D == 3 ? 4 : 3) :
 
         // ---------------- phase 4: divergence and output ----------------
         const double dt = L.mode == MODE_RK ? *P.dt : 0.0;
-        for (int t = threadIdx.x; t < S * WT; t += blockDim.x) {
+        for (int t = threadIdx.x; t < sE * wE; t += blockDim.x) {
             int s, w;
-            if (k == 0) { s = t % S; w = t / S; }
-            else { w = t % WT; s = t / WT; }
+            if (k == 0) { w = div_small(t, rS); s = t - w * sE; }
+            else { s = div_small(t, rW); w = t - s * wE; }
             const int g = s0 + s, a = a0 + w;
-            if (g >= nk || a >= na) continue;
             int idx[3] = { 0, 0, 0 };
             idx[k] = g;
             idx[adim] = a;
@@ -267,45 +281,74 @@ static size_t smem_of()
     return stage_offset<D, NS, R, S, WT>() + (stages_inputs<D, NS>() ? sizeof(double) * stage_rows<D, NS>() * Tile<S, WT>::NN : 0);
 }
 
-// one case per tile shape of the table in es_kernels.cuh
+// one case per tile shape of the table in es_kernels.cuh; 3D FP64: the run-time extent
 #define ES_FLUX_SHAPES(X) X(0) X(1) X(2) X(3) X(4) X(5)
 static_assert(NSHAPE == 6, "ES_FLUX_SHAPES lists every tile shape");
+
+template <int D, typename R>
+__host__ __device__ constexpr bool fits_tiles() { return D == 3 && std::is_same<R, double>::value; }
+
+template <int D, int NS, typename R, int S, int WT, int WK>
+static void prepare_shape()
+{
+    cudaFuncSetAttribute(flux_kernel<D, NS, R, S, WT, WK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)smem_of<D, NS, R, S, WT>());
+}
 
 template <int D, int NS, typename R, int WK>
 void prepare_flux()
 {
-#define ES_PREP(SH)                                                                                       \
-    cudaFuncSetAttribute(flux_kernel<D, NS, R, SHAPE_S[SH], SHAPE_WT[SH], WK>,                             \
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_of<D, NS, R, SHAPE_S[SH], SHAPE_WT[SH]>());
-    ES_FLUX_SHAPES(ES_PREP)
+    if constexpr (fits_tiles<D, R>()) {
+        prepare_shape<D, NS, R, 0, 0, WK>();
+    } else {
+#define ES_PREP(SH) prepare_shape<D, NS, R, SHAPE_S[SH], SHAPE_WT[SH], WK>();
+        ES_FLUX_SHAPES(ES_PREP)
 #undef ES_PREP
+    }
+}
+
+template <int D, int NS, typename R, int S, int WT, int WK>
+static int shape_blocks()
+{
+    int nb = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, flux_kernel<D, NS, R, S, WT, WK>, FLUX_TPB, smem_of<D, NS, R, S, WT>());
+    return nb > 0 ? nb : 1;
 }
 
 template <int D, int NS, typename R, int WK>
 int flux_blocks_per_sm(int shape)
 {
-    int nb = 0;
-#define ES_OCC(SH)                                                                                           \
-    if (shape == SH)                                                                                         \
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, flux_kernel<D, NS, R, SHAPE_S[SH], SHAPE_WT[SH], WK>, \
-                                                      FLUX_TPB, smem_of<D, NS, R, SHAPE_S[SH], SHAPE_WT[SH]>());
-    ES_FLUX_SHAPES(ES_OCC)
+    if constexpr (fits_tiles<D, R>()) {
+        (void)shape;
+        return shape_blocks<D, NS, R, 0, 0, WK>();
+    } else {
+#define ES_OCC(SH) if (shape == SH) return shape_blocks<D, NS, R, SHAPE_S[SH], SHAPE_WT[SH], WK>();
+        ES_FLUX_SHAPES(ES_OCC)
 #undef ES_OCC
-    return nb > 0 ? nb : 1;
+        return 1;
+    }
+}
+
+template <int D, int NS, typename R, int S, int WT, int WK>
+static void launch_shape(const FluxLaunch& L, int grid, cudaStream_t st)
+{
+    // the staging buffer only when a CTA has several tiles (the kernel's own test)
+    const bool staged = stages_inputs<D, NS>() && L.nwork > grid;
+    pdl_launch(flux_kernel<D, NS, R, S, WT, WK>, grid, FLUX_TPB,
+               staged ? smem_of<D, NS, R, S, WT>() : stage_offset<D, NS, R, S, WT>(), st, L);
 }
 
 template <int D, int NS, typename R, int WK>
 void launch_flux(const FluxLaunch& L, int shape, int grid, cudaStream_t st)
 {
-    // the staging buffer only when a CTA has several tiles (the kernel's own test)
-    const bool staged = stages_inputs<D, NS>() && L.nwork > grid;
-#define ES_LAUNCH(SH)                                                                                        \
-    if (shape == SH)                                                                                         \
-        pdl_launch(flux_kernel<D, NS, R, SHAPE_S[SH], SHAPE_WT[SH], WK>, grid, FLUX_TPB,                       \
-                   staged ? smem_of<D, NS, R, SHAPE_S[SH], SHAPE_WT[SH]>() : stage_offset<D, NS, R, SHAPE_S[SH], SHAPE_WT[SH]>(), \
-                   st, L);
-    ES_FLUX_SHAPES(ES_LAUNCH)
+    if constexpr (fits_tiles<D, R>()) {
+        (void)shape;
+        launch_shape<D, NS, R, 0, 0, WK>(L, grid, st);
+    } else {
+#define ES_LAUNCH(SH) if (shape == SH) launch_shape<D, NS, R, SHAPE_S[SH], SHAPE_WT[SH], WK>(L, grid, st);
+        ES_FLUX_SHAPES(ES_LAUNCH)
 #undef ES_LAUNCH
+    }
 }
 
 // explicit instantiation of one (dimension, species, reconstruction) case in both compute types

@@ -7,8 +7,11 @@ namespace es {
 
 // flux tile shapes: S nodes along the line x WT neighbouring lines, (S + 1) WT <= 256
 // interfaces (one thread each), (S + 6) WT staged nodes and (3S + 6) WT distinct node pairs.
-// The autotuner picks one shape (and a persistent grid size) per direction.
+// The autotuner picks one shape (and a persistent grid size) per direction; a 3D context that
+// nobody tuned picks by its grid (pick_tiles_3d in es_api.cu), the FP64 form any extent within
+// those limits.
 constexpr int FLUX_TPB = 256;
+constexpr int FLUX_WT_MAX = 16;
 constexpr int NSHAPE = 6;
 constexpr int SHAPE_S[NSHAPE] = { 62, 58, 122, 30, 26, 14 };
 constexpr int SHAPE_WT[NSHAPE] = { 4, 4, 2, 8, 8, 16 };
@@ -57,6 +60,7 @@ struct FluxLaunch {
     const int2* work;
     int nwork;
     int k;             // direction (per-direction kernel)
+    int S, WT;         // 3D FP64: the tile's nodes along the line and lines (else by shape)
     int mode;          // MODE_*
     double a, b;       // Shu-Osher coefficients of the stage (MODE_RK)
     double mcoef;      // 2D: the stage metrics are M + mcoef dt Md (0: M alone)

@@ -590,3 +590,22 @@ def test_integer_pipe_conversions_match_hardware():
     assert bool(torch.isnan(o32[nan]).all()) and bool(torch.isnan(o64[nan]).all())
     assert torch.equal(o64[~nan], o32[~nan].double())
     assert bool((o32[~keep & ~nan] == 0).all())
+
+
+@pytest.mark.parametrize("form", [0, 1])
+@pytest.mark.parametrize("N,n", [(1, (63, 17, 10)), (1, (33, 10, 31)), (2, (124, 11, 13)), (2, (10, 10, 64))])
+def test_untuned_3d_tiles_bitwise(form, N, n):
+    """The tiles that an untuned 3D context picks by its grid (in the FP64 form of any extent) give
+    the residual of every shape of the table bit for bit, with one-node and nearly full partial
+    tiles at the ends of the lines."""
+    torch = need_gpu()
+    pb, JU, J, x, xdot = case(3, N, n, "mixed", es=True, seed=71 + N, jump=True)
+    G = [to_dev(t, torch) for t in (JU, J, x, xdot)]
+    ctx = _ctx(pb, form)
+    ref = ctx.es_rhs(*G)
+    assert all((S + 1) * WT <= 256 and S > 0 for _, S, WT, _, _ in ctx.es_get_tuning())
+    for shape in range(6):
+        for k in range(3):
+            ctx.es_set_tuning(k, shape)
+        got = ctx.es_rhs(*G)
+        assert torch.equal(got[0], ref[0]) and torch.equal(got[1], ref[1]), shape
