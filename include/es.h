@@ -198,10 +198,10 @@ es_status es_set_tuning(es_ctx* ctx, int k, int shape, int grid);
  * results are bitwise those of the per-direction launches.  es_autotune on a 2D
  * context also times each fused shape and keeps the fused launch when it beats
  * the sum of the best per-direction launches.  A new 2D context starts with the
- * fused launch in shape 0 (16 x 12 tiles, full occupancy).  On grids of few tiles
- * a new context, and es_autotune where it measures them faster, run the launch on
- * smaller tiles (8 x 8, 12 x 8 or 16 x 8) behind the reported shape; a shape set by
- * es_set_fusion runs as it is.
+ * fused launch in shape 0 (16 x 12 tiles, full occupancy).  A new context by its
+ * grid, and es_autotune where it measures them faster, run the launch on other
+ * tiles behind the reported shape (8 x 8, 12 x 8 or 16 x 8 on grids of few tiles;
+ * 16 x 14 or 24 x 15 in the FP64 form); a shape set by es_set_fusion runs as it is.
  * es_get_fusion: fused shape index (-1: per-direction launches), TX, TY, grid
  * (CTAs) and the best fused time per launch the last es_autotune measured (0 if
  * none; set even when the per-direction launches won).  All pointers HOST, one

@@ -338,7 +338,7 @@ void pick_fused(es_ctx* c)
     c->fused_run = -1;
     double best = 0.0;
     for (int sh = 0; sh < NFSHAPE_ALL; ++sh) {
-        if (sh > 0 && sh < NFSHAPE) continue;
+        if ((sh > 0 && sh < NFSHAPE) || (c->mixed && sh >= NFSHAPE_MIXED)) continue;
         const int slots = c->sms * flux2d_occ(c, sh);
         const double cost = (double)((c->n_fused[sh] + slots - 1) / slots) * FSHAPE_COST[sh][c->mixed ? 0 : 1];
         if (sh == 0 || cost < best) {
@@ -1274,9 +1274,9 @@ es_status es_autotune(es_ctx* c, const double* JU, const double* J, const double
     c->fused_ms = 0.f;
     drop_run_graph(c);
     if (c->d == 2) {
-        // the small-grid shapes last: they take over the launch, not the reported shape
+        // the shapes beyond the table last: they take over the launch, not the reported shape
         float best = 3.0e38f;
-        for (int sh = 0; sh < NFSHAPE_ALL; ++sh) {
+        for (int sh = 0; sh < (c->mixed ? NFSHAPE_MIXED : NFSHAPE_ALL); ++sh) {
             const int occ = flux2d_occ(c, sh);
             for (int o = occ; o >= 1 && o >= occ - 1; --o) {
                 FluxLaunch L;

@@ -227,16 +227,19 @@ __global__ void __launch_bounds__(FLUX_TPB, (sizeof(R) == 4 ? 3 : 1)) flux2d_ker
     }
 }
 
-// one case per fused tile shape of the table in es_kernels.cuh
-#define ES_FLUX2D_SHAPES(X) X(0) X(1) X(2) X(3) X(4) X(5) X(6) X(7)
-static_assert(NFSHAPE_ALL == 8, "ES_FLUX2D_SHAPES lists every fused tile shape");
+// one case per fused tile shape of the table in es_kernels.cuh (the binary32 kernels lack the last)
+#define ES_FLUX2D_SHAPES(X) X(0) X(1) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9)
+static_assert(NFSHAPE_ALL == 10, "ES_FLUX2D_SHAPES lists every fused tile shape");
+template <typename R, int SH>
+constexpr bool has_fshape() { return SH < NFSHAPE_MIXED || std::is_same<R, double>::value; }
 
 template <int NS, typename R, int WK>
 void prepare_flux2d()
 {
 #define ES_PREP2(SH)                                                                                        \
-    cudaFuncSetAttribute(flux2d_kernel<NS, R, FSHAPE_TX[SH], FSHAPE_TY[SH], WK>,                             \
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_flux2d<NS, R, FSHAPE_TX[SH], FSHAPE_TY[SH]>());
+    if constexpr (has_fshape<R, SH>())                                                                      \
+        cudaFuncSetAttribute(flux2d_kernel<NS, R, FSHAPE_TX[SH], FSHAPE_TY[SH], WK>,                         \
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_flux2d<NS, R, FSHAPE_TX[SH], FSHAPE_TY[SH]>());
     ES_FLUX2D_SHAPES(ES_PREP2)
 #undef ES_PREP2
 }
@@ -246,9 +249,10 @@ int flux2d_blocks_per_sm(int shape)
 {
     int nb = 0;
 #define ES_OCC2(SH)                                                                                            \
-    if (shape == SH)                                                                                           \
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, flux2d_kernel<NS, R, FSHAPE_TX[SH], FSHAPE_TY[SH], WK>, \
-                                                      FLUX_TPB, smem_flux2d<NS, R, FSHAPE_TX[SH], FSHAPE_TY[SH]>());
+    if constexpr (has_fshape<R, SH>())                                                                         \
+        if (shape == SH)                                                                                       \
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, flux2d_kernel<NS, R, FSHAPE_TX[SH], FSHAPE_TY[SH], WK>, \
+                                                          FLUX_TPB, smem_flux2d<NS, R, FSHAPE_TX[SH], FSHAPE_TY[SH]>());
     ES_FLUX2D_SHAPES(ES_OCC2)
 #undef ES_OCC2
     return nb > 0 ? nb : 1;
@@ -258,9 +262,10 @@ template <int NS, typename R, int WK>
 void launch_flux2d(const FluxLaunch& L, int shape, int grid, cudaStream_t st)
 {
 #define ES_LAUNCH2(SH)                                                                                        \
-    if (shape == SH)                                                                                          \
-        pdl_launch(flux2d_kernel<NS, R, FSHAPE_TX[SH], FSHAPE_TY[SH], WK>, grid, FLUX_TPB,                    \
-                   smem_flux2d<NS, R, FSHAPE_TX[SH], FSHAPE_TY[SH]>(), st, L);
+    if constexpr (has_fshape<R, SH>())                                                                        \
+        if (shape == SH)                                                                                      \
+            pdl_launch(flux2d_kernel<NS, R, FSHAPE_TX[SH], FSHAPE_TY[SH], WK>, grid, FLUX_TPB,                \
+                       smem_flux2d<NS, R, FSHAPE_TX[SH], FSHAPE_TY[SH]>(), st, L);
     ES_FLUX2D_SHAPES(ES_LAUNCH2)
 #undef ES_LAUNCH2
 }

@@ -289,10 +289,11 @@ def test_mesh_sweeps_in_several_launches(bc, mu, nf):
 
 
 @pytest.mark.parametrize("form", [0, 1])
-@pytest.mark.parametrize("N,n,weno", [(1, (10, 11), 0), (1, (64, 64), 0), (2, (81, 41), 1), (2, (150, 75), 0), (1, (128, 121), 0)])
+@pytest.mark.parametrize("N,n,weno", [(1, (10, 11), 0), (1, (64, 64), 0), (2, (81, 41), 1), (2, (150, 75), 0), (1, (128, 121), 0),
+                                      (2, (255, 241), 0), (2, (349, 151), 0)])
 def test_small_grid_tiles_bitwise(form, N, n, weno):
-    """The tiles that an untuned context takes on a small grid (8 x 8, 12 x 8 and 16 x 8, with
-    ragged edges) give the residual and the RK step of the 16 x 12 tiles bit for bit."""
+    """The tiles that an untuned context takes by its grid (8 x 8, 12 x 8 and 16 x 8 on small ones,
+    16 x 14 and 24 x 15 in the FP64 form, with ragged edges) give the residual and the RK step of the 16 x 12 tiles bit for bit."""
     torch = need_gpu()
     pb, JU, J, x, xdot = case(2, N, n, "mixed", es=True, seed=51 + N, jump=True)
     pb = pb.with_(weno=weno)
