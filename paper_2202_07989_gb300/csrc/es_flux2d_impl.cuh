@@ -28,6 +28,13 @@ struct Tile2 {
     static constexpr int NI0 = (TX + 1) * TY, NI1 = (TY + 1) * TX;
     static constexpr int NI = NI0 > NI1 ? NI0 : NI1;
     static constexpr int NM0 = (TX + 6) * TY, NM1 = TX * (TY + 6);   // FP64 J xi_k/t on the rows / columns
+    // Small tiles run both directions in the same phases: their interfaces, 72 + 72 of an 8 x 8
+    // tile, leave most of the 256 threads idle one direction at a time, and such a launch lasts as
+    // long as one tile's chain of phases.  Whole warps take one direction, and each direction has
+    // its own pair, mean and flux arrays (64^2, 8 x 8 tiles: FP64 launch 74 -> 64 us, mixed residual
+    // 17.0 -> 15.6 us).
+    static constexpr bool BOTH = (NI0 + 31) / 32 * 32 + NI1 <= FLUX_TPB && NO <= FLUX_TPB / 2;
+    static constexpr int ND = BOTH ? 2 : 1;
 };
 
 template <int NS, typename R, int TX, int TY>
@@ -35,8 +42,8 @@ __host__ __device__ constexpr size_t smem_flux2d()
 {
     using Y = Lay<2, NS>;
     using T = Tile2<TX, TY>;
-    return sizeof(double) * ((Y::NC + 1) * T::NO + T::NI + T::NM0 + T::NM1) +
-           sizeof(R) * ((Y::NF + 3) * T::NN + Y::NC * T::NP + (NS + 1) * T::NI + Y::NC * T::NI);
+    return sizeof(double) * ((T::BOTH ? 0 : (Y::NC + 1) * T::NO) + T::ND * T::NI + T::NM0 + T::NM1) +
+           sizeof(R) * ((Y::NF + 3) * T::NN + T::ND * (Y::NC * T::NP + (NS + 1) * T::NI + Y::NC * T::NI));
 }
 
 // Phases 2 (distinct pairs) and 3 (interfaces) of direction K (0: along the rows, 1: along
@@ -45,14 +52,15 @@ __host__ __device__ constexpr size_t smem_flux2d()
 // consecutive nodes in both directions.  The kernel inlines both directions (constant K);
 // a single copy looping over a run-time K measured no faster.
 template <int NS, typename R, int TX, int TY, int WK>
-__device__ __forceinline__ void flux2d_pairs(const int K, const Inst& I, int i0, int j0, const R* nr, R* pf, R* cm)
+__device__ __forceinline__ void flux2d_pairs(const int K, const Inst& I, int i0, int j0, const R* nr, R* pf, R* cm,
+                                             int first, int step)
 {
     using Y = Lay<2, NS>;
     using T = Tile2<TX, TY>;
     constexpr int NN = T::NN, NP = T::NP, NI = T::NI, RW = T::RW;
     const int S = K ? TY : TX, NPK = K ? T::NP1 : T::NP0, MR = K ? Y::NF : Y::MR;
     const int nk = I.n[K], na = I.n[1 - K], s0 = K ? j0 : i0, a0 = K ? i0 : j0;
-    for (int t = threadIdx.x; t < NPK; t += blockDim.x) {
+    for (int t = first; t < NPK; t += step) {
         const int w = K ? t % TX : t / T::NPL0, r_ = K ? t / TX : t % T::NPL0;
         int m, Ln;
         if (r_ < S + 1) { m = 1; Ln = r_ + 2; }
@@ -67,7 +75,7 @@ __device__ __forceinline__ void flux2d_pairs(const int K, const Inst& I, int i0,
 
 template <int NS, typename R, int TX, int TY, int WK>
 __device__ __forceinline__ void flux2d_ifaces(const int K, const Inst& I, int i0, int j0, const R* nr, const double* mtk,
-                                              const R* pf, const R* cm, R* fl, double* gt)
+                                              const R* pf, const R* cm, R* fl, double* gt, int first, int step)
 {
     using Y = Lay<2, NS>;
     using T = Tile2<TX, TY>;
@@ -76,7 +84,7 @@ __device__ __forceinline__ void flux2d_ifaces(const int K, const Inst& I, int i0
     const int nk = I.n[K], na = I.n[1 - K], s0 = K ? j0 : i0, a0 = K ? i0 : j0;
     // strides: nodes along the line, J xi_k/t along the line, pairs of one kind along the line
     const int ns = K ? RW : 1, ms = K ? TX : 1, ps = K ? TX : 1;
-    for (int f = threadIdx.x; f < NIK; f += blockDim.x) {
+    for (int f = first; f < NIK; f += step) {
         const int w = K ? f % TX : f / (TX + 1), s = K ? f / TX : f % (TX + 1);
         const int gi = s0 - 1 + s;     // interface gi + 1/2
         if (a0 + w >= na || gi > nk - 1) continue;
@@ -115,13 +123,13 @@ __global__ void __launch_bounds__(FLUX_TPB, (sizeof(R) == 4 ? 3 : 1)) flux2d_ker
     constexpr int NC = Y::NC, NN = T::NN, NI = T::NI, NP = T::NP, NO = T::NO, RW = T::RW;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double* acc = reinterpret_cast<double*>(smem_raw);      // [NC + 1][NO] divergence of direction 1
-    double* gt = acc + (NC + 1) * NO;                       // [NI] GCL flux of J xi_k/t
-    double* mt0 = gt + NI;                                  // [TY][TX + 6] J xi_1/t on the rows
+    double* gt = acc + (T::BOTH ? 0 : (NC + 1) * NO);       // [ND][NI] GCL flux of J xi_k/t
+    double* mt0 = gt + T::ND * NI;                              // [TY][TX + 6] J xi_1/t on the rows
     double* mt1 = mt0 + T::NM0;                             // [TY + 6][TX] J xi_2/t on the columns
     R* nr = reinterpret_cast<R*>(mt1 + T::NM1);             // [NF + 3][NN] node data, both metric rows
-    R* pf = nr + (Y::NF + 3) * NN;                          // [NC][NP] pair fluxes
-    R* cm = pf + NC * NP;                                   // [NS + 1][NI] centre-pair means
-    R* fl = cm + (NS + 1) * NI;                             // [NC][NI] interface fluxes
+    R* pf = nr + (Y::NF + 3) * NN;                          // [ND][NC][NP] pair fluxes
+    R* cm = pf + T::ND * NC * NP;                           // [ND][NS + 1][NI] centre-pair means
+    R* fl = cm + T::ND * (NS + 1) * NI;                     // [ND][NC][NI] interface fluxes
 
     for (int wi = blockIdx.x; wi < L.nwork; wi += gridDim.x) {
         const int2 it = L.work[wi];
@@ -191,18 +199,35 @@ __global__ void __launch_bounds__(FLUX_TPB, (sizeof(R) == 4 ? 3 : 1)) flux2d_ker
         }
         __syncthreads();
 
+        const int tid = (int)threadIdx.x;
+        if constexpr (T::BOTH) {
+            // ---------------- both directions: pairs, then interfaces ----------------
+            // (the directions' items in turn, each starting at a warp)
+            constexpr int P0 = (T::NP0 + 31) / 32 * 32, F0 = (T::NI0 + 31) / 32 * 32;
+            for (int t = tid; t < P0 + T::NP1; t += FLUX_TPB) {
+                if (t < P0) flux2d_pairs<NS, R, TX, TY, WK>(0, I, i0, j0, nr, pf, cm, t, T::NP0);
+                else flux2d_pairs<NS, R, TX, TY, WK>(1, I, i0, j0, nr, pf + NC * NP, cm + (NS + 1) * NI, t - P0, T::NP1);
+            }
+            __syncthreads();
+            if (tid < F0) flux2d_ifaces<NS, R, TX, TY, WK>(0, I, i0, j0, nr, mt0, pf, cm, fl, gt, tid, T::NI0);
+            else
+                flux2d_ifaces<NS, R, TX, TY, WK>(1, I, i0, j0, nr, mt1, pf + NC * NP, cm + (NS + 1) * NI, fl + NC * NI,
+                                                 gt + NI, tid - F0, T::NI1);
+            __syncthreads();
+        } else {
         // ---------------- direction 1: pairs, interfaces ----------------
-        flux2d_pairs<NS, R, TX, TY, WK>(0, I, i0, j0, nr, pf, cm);
+        flux2d_pairs<NS, R, TX, TY, WK>(0, I, i0, j0, nr, pf, cm, tid, FLUX_TPB);
         __syncthreads();
-        flux2d_ifaces<NS, R, TX, TY, WK>(0, I, i0, j0, nr, mt0, pf, cm, fl, gt);
+        flux2d_ifaces<NS, R, TX, TY, WK>(0, I, i0, j0, nr, mt0, pf, cm, fl, gt, tid, FLUX_TPB);
         __syncthreads();
 
         // ---------------- divergence of direction 1; direction 2: pairs, interfaces ----------------
         flux2d_div1<NS, R, TX, TY>(I, i0, j0, fl, gt, acc);
-        flux2d_pairs<NS, R, TX, TY, WK>(1, I, i0, j0, nr, pf, cm);
+        flux2d_pairs<NS, R, TX, TY, WK>(1, I, i0, j0, nr, pf, cm, tid, FLUX_TPB);
         __syncthreads();
-        flux2d_ifaces<NS, R, TX, TY, WK>(1, I, i0, j0, nr, mt1, pf, cm, fl, gt);
+        flux2d_ifaces<NS, R, TX, TY, WK>(1, I, i0, j0, nr, mt1, pf, cm, fl, gt, tid, FLUX_TPB);
         __syncthreads();
+        }
 
         // ---------------- divergence of direction 2 and output ----------------
         const double dt = L.mode == MODE_RK ? *P.dt : 0.0;
@@ -210,17 +235,26 @@ __global__ void __launch_bounds__(FLUX_TPB, (sizeof(R) == 4 ? 3 : 1)) flux2d_ker
             const int il = t % TX, jl = t / TX;
             if (i0 + il >= n0 || j0 + jl >= n1) continue;
             const long long id = lin(I, i0 + il, j0 + jl, 0);
-            double r[NC + 1];
-            node_div<NC, R>(I, fl, NI, gt, t + TX, t, 1, r);
+            // both directions' divergences, r_1 + r_2
+            double r[NC + 1], r1[NC + 1];
+            if constexpr (T::BOTH) {
+                const int fr = jl * (TX + 1) + il + 1;
+                node_div<NC, R>(I, fl, NI, gt, fr, fr - 1, 0, r1);
+                node_div<NC, R>(I, fl + NC * NI, NI, gt + NI, t + TX, t, 1, r);
+            } else {
+#pragma unroll
+                for (int q = 0; q <= NC; ++q) r1[q] = acc[q * NO + t];
+                node_div<NC, R>(I, fl, NI, gt, t + TX, t, 1, r);
+            }
             if (L.mode == MODE_RK) {
 #pragma unroll
                 for (int q = 0; q < NC; ++q)
-                    P.JUo[q * ncell + id] = rk_stage(L, P.JU[q * ncell + id], P.JU0 + q * ncell + id, dt, acc[q * NO + t] + r[q]);
-                P.Jo[id] = rk_stage(L, P.J[id], P.J0 + id, dt, acc[NC * NO + t] + r[NC]);
+                    P.JUo[q * ncell + id] = rk_stage(L, P.JU[q * ncell + id], P.JU0 + q * ncell + id, dt, r1[q] + r[q]);
+                P.Jo[id] = rk_stage(L, P.J[id], P.J0 + id, dt, r1[NC] + r[NC]);
             } else {
 #pragma unroll
-                for (int q = 0; q < NC; ++q) P.accU[q * ncell + id] = acc[q * NO + t] + r[q];
-                P.accJ[id] = acc[NC * NO + t] + r[NC];
+                for (int q = 0; q < NC; ++q) P.accU[q * ncell + id] = r1[q] + r[q];
+                P.accJ[id] = r1[NC] + r[NC];
             }
         }
         __syncthreads();

@@ -22,8 +22,8 @@ constexpr int SHAPE_DEFAULT_KN = 3;    // directions 2, 3: 30 nodes x 8 neighbou
 // shapes from NFSHAPE on are for small grids: a grid of few tiles is bound by the time one tile
 // takes, not by the chip, and a smaller tile takes less.  FSHAPE_COST is the time of one wave of
 // CTAs in each shape relative to 16 x 12 tiles, binary32 and binary64, measured on grids of one wave
-// (single-species FP64 launches, us: 16 x 12 139.6, 8 x 8 73.7, 12 x 8 85.9, 16 x 8 110, 16 x 14 158,
-// 24 x 15 237; mixed residuals 21.6, 17.0, 17.8, 19.4), by which a context that nobody tuned
+// (single-species FP64 launches, us: 16 x 12 139.6, 8 x 8 64, 12 x 8 82, 16 x 8 110, 16 x 14 158,
+// 24 x 15 237; mixed residuals, metrics pass included, 21.9, 15.6, 16.3, 19.5), by which a context that nobody tuned
 // picks its tiles: the least waves x cost (pick_fused in es_api.cu).
 constexpr int NFSHAPE = 5;
 // The last two are for the FP64 form only, whose phases cost whole warps on each of the SM's four
@@ -34,7 +34,7 @@ constexpr int NFSHAPE_ALL = 10, NFSHAPE_MIXED = 8;
 constexpr int FSHAPE_TX[NFSHAPE_ALL] = { 16, 12, 14, 24, 20, 8, 12, 16, 16, 24 };
 constexpr int FSHAPE_TY[NFSHAPE_ALL] = { 12, 16, 14, 8, 10, 8, 8, 8, 14, 15 };
 constexpr double FSHAPE_COST[NFSHAPE_ALL][2] = { { 1.0, 1.0 }, { 1.0, 1.0 }, { 1.0, 1.0 }, { 1.0, 1.0 }, { 1.0, 1.0 },
-                                                 { 0.75, 0.52 }, { 0.8, 0.61 }, { 0.88, 0.79 }, { 0.0, 1.13 }, { 0.0, 1.7 } };
+                                                 { 0.71, 0.46 }, { 0.74, 0.59 }, { 0.88, 0.79 }, { 0.0, 1.13 }, { 0.0, 1.7 } };
 constexpr int NODE_TPB = 256;
 
 // launch with programmatic stream serialization (the kernel must begin with pdl_entry())
