@@ -215,29 +215,31 @@ __device__ __forceinline__ double min_pos(double a, double b)
 
 // WENO-MR (Appendix A) of the FP64 form from the node differences D_m = W_{j-1+m} - W_{j-2+m}
 // (m = 0..3): the value at x_{j+1/2} is W_j + num / den, for linear weights that sum to one.
-// The indicators, candidate values and weights of weno_mr, written in s = D1 + D2, e = D2 - D1,
-// t = D0 + D3, u = D3 - D0 and cleared of the common denominator: t_1 = (7s - t)/12, t_2 =
-// (163e - 11u)/260, b_4 = (t - s)/12, b_5 = (u - 3e)/24, h_2 - W_j = s/4 + e/12, h_3 - W_j =
-// (-2 D0 + 11 D1 + 24 D2 - 3 D3)/60.  All differences of W, so nothing cancels against W itself.
-// Why: the FP64 form is bound by its pipe, and this takes about 50 FP64 instructions and no
+// The indicators, candidate values and weights of weno_mr in s = D1 + D2, e = D2 - D1, t = D0 +
+// D3, u = D3 - D0: beta_2 = s^2/4 + 13 e^2/12; beta_3, whose even part depends on (s, t) and its odd
+// part on (e, u), with both squares completed; h_2 - W_j = s/4 + e/12, h_3 - W_j = (-2 D0 + 11 D1 +
+// 24 D2 - 3 D3)/60; and with E_k = eps + beta_k, Pi = E_1 E_2 E_3 and tau, the weights times Pi are
+// chi_1 (Pi + tau E_2 E_3) and so on, whose sum is Pi + tau (chi_1 E_2 E_3 + chi_2 E_1 E_3 + chi_3 E_1
+// E_2).  All differences of W, so nothing cancels against W itself.
+// Why: the FP64 form is bound by its pipe, and this takes about 41 FP64 instructions and no
 // division where weno_mr takes about 80 with one; W^+ mirrors to the same function of the
 // negated differences, so the jump needs one division for both (weno_mr_jump).
 __device__ __forceinline__ void weno_mr_corr(double D0, double D1, double D2, double D3, double q1, double q2, double c1,
                                              double c2, double c3, double eps, double& num, double& den)
 {
-    const double s = D1 + D2, e = D2 - D1, t = D0 + D3, u = D3 - D0, h = 0.5 * s;
+    const double s = D1 + D2, e = D2 - D1, t = D0 + D3, u = D3 - D0;
+    const double ss = __dmul_rn(s, s), ee = __dmul_rn(e, e);
     const double E1 = eps + min_pos(q1, q2);
-    const double E2 = fma((13.0 / 12.0) * e, e, fma(h, h, eps));
-    const double A = fma(7.0, s, -t), P = t - s, B = fma(-11.0 / 163.0, u, e), r = fma(-3.0, e, u);
-    const double E3 = fma((1.0 / 144.0) * A, A, fma((781.0 / 2880.0) * P, P, fma((26569.0 / 15600.0) * B, B,
-                      fma((1421461.0 / 1310400.0) * r, r, eps))));
-    const double x = fabs(E3 - E1) + fabs(E3 - E2), X = x * x;     // tau = X / 4
-    const double f1 = fma(0.25, X, E1), f2 = fma(0.25, X, E2), f3 = fma(0.25, X, E3);
-    const double h2 = fma(1.0 / 12.0, e, 0.5 * h);
+    const double E2 = fma(0.25, ss, fma(13.0 / 12.0, ee, eps));
+    const double v = fma(-307.0 / 267.0, s, t), z = fma(-67923.0 / 22025.0, e, u);
+    const double E3 = fma((89.0 / 320.0) * v, v, fma(781.0 / 3204.0, ss,
+                      fma((4405.0 / 4032.0) * z, z, fma(1421461.0 / 1321500.0, ee, eps))));
+    const double x = fabs(E3 - E1) + fabs(E3 - E2), tau = 0.25 * x * x;
+    const double g = fma(c2 * (1.0 / 12.0), e, (c2 * 0.25) * s);       // chi_2 (h_2 - W_j)
     const double h3 = fma(24.0 / 60.0, D2, fma(11.0 / 60.0, D1, fma(-3.0 / 60.0, D3, (-2.0 / 60.0) * D0)));
-    const double o1 = __dmul_rn(c1 * f1, E2 * E3), o2 = __dmul_rn(c2 * f2, E1 * E3), o3 = __dmul_rn(f3, E1 * E2);
-    den = fma(c3, o3, o1 + o2);
-    num = fma(o2, h2, __dmul_rn(o3, fma(-c2, h2, h3)));
+    const double E12 = __dmul_rn(E1, E2), E13 = __dmul_rn(E1, E3), E23 = __dmul_rn(E2, E3), Pi = __dmul_rn(E12, E3);
+    den = fma(tau, fma(c1, E23, fma(c2, E13, __dmul_rn(c3, E12))), Pi);
+    num = fma(g, fma(tau, E13, Pi), __dmul_rn(h3 - g, fma(tau, E12, Pi)));
 }
 
 // [[W]]^WENO-MR at the interface from the five node differences D_0..D_4 of its stencil
@@ -597,7 +599,10 @@ __device__ __forceinline__ void iface_flux(const Inst& I, const R* nb, int NN, i
     }
     // GCL flux of (J xi_k/t, J xi_k/x_j): stencil (1, -8, 37, 37, -8, 1)/60 for w = 3
     const double c0 = I.gcw[0], c1 = I.gcw[1], c2 = I.gcw[2];
-    const double Gt = mad(c2, m64[0] + m64[5 * ms], dot2(c0, m64[2 * ms] + m64[3 * ms], c1, m64[ms] + m64[4 * ms]));
+    double Gt;
+    if constexpr (std::is_same<R, double>::value)
+        Gt = mad(c2, m64[0] + m64[5 * ms], dot2(c0, m64[2 * ms] + m64[3 * ms], c1, m64[ms] + m64[4 * ms]));
+    else Gt = c0 * (m64[2 * ms] + m64[3 * ms]) + c1 * (m64[ms] + m64[4 * ms]) + c2 * (m64[0] + m64[5 * ms]);
     gt[f] = Gt;
     if (I.es) {
         R Gx[D], L2 = R(0);
@@ -900,14 +905,18 @@ __device__ __forceinline__ void node_div(const Inst& I, const R* fl, int NI, con
     R rdx;
     if constexpr (std::is_same<R, float>::value) rdx = I.f_inv_dxi[k];
     else rdx = inv_dx;
-    r[NC] = __dmul_rn(-(gt[fr] - gt[fL]), inv_dx);
+    if constexpr (std::is_same<R, double>::value) {
+        // (rounded products: the sums over the directions start from them)
+        r[NC] = __dmul_rn(-(gt[fr] - gt[fL]), inv_dx);
 #pragma unroll
-    for (int q = 0; q < NC; ++q) {
-        // (a rounded product: the sums over the directions start from it)
-        if constexpr (std::is_same<R, double>::value) r[q] = __dmul_rn(-(fl[q * NI + fr] - fl[q * NI + fL]), rdx);
-        else r[q] = to_d(-(fl[q * NI + fr] - fl[q * NI + fL]) * rdx);
+        for (int q = 0; q < NC; ++q) r[q] = __dmul_rn(-(fl[q * NI + fr] - fl[q * NI + fL]), rdx);
+        r[NC - 1] = fma(I.pinf_tot, r[NC], r[NC - 1]);
+    } else {
+        r[NC] = -(gt[fr] - gt[fL]) * inv_dx;
+#pragma unroll
+        for (int q = 0; q < NC; ++q) r[q] = to_d(-(fl[q * NI + fr] - fl[q * NI + fL]) * rdx);
+        r[NC - 1] += I.pinf_tot * r[NC];
     }
-    r[NC - 1] = fma(I.pinf_tot, r[NC], r[NC - 1]);
 }
 
 }  // namespace es
