@@ -567,6 +567,10 @@ void launch_residual(es_ctx* c, const StagePtrs& P, const StagePtrs* tab, bool r
         flux2d_launch(c, L, sh, c->fused_run >= 0 ? c->fused_run_grid : c->fused_grid, st);
         return;
     }
+    if (c->d == 3 && c->mixed) {
+        ProfScope ps(c, PC_FLUX, st);
+        launch_prim3d(c->N, node_grid(c, c->n_cell), st, c->dI, P, tab, c->w_cell, c->n_cell, c->status);
+    }
     for (int k = 0; k < c->d; ++k) {
         FluxLaunch L;
         L.insts = c->dI;
@@ -623,6 +627,7 @@ void stage_ptrs(es_ctx* c, int i, double* JU, double* J, double* x, const double
         // step's mesh) in M and forms the third stage's in M3
         P.M = (s == 2 && S.M3) ? S.M3 : S.M;
         P.Md = S.Md;
+        P.prim = S.prim;
         P.accU = S.accU;
         P.accJ = S.accJ;
         P.JU0 = JU;
@@ -817,6 +822,7 @@ es_status es_create_batch(const es_config* cfgs, int n_inst, es_ctx** out)
         long long n = I.ncell;
         ok = ok && dalloc(c, (void**)&S.M, sizeof(double) * I.d * (I.d + 1) * I.npad);
         if (I.d == 2) ok = ok && dalloc(c, (void**)&S.Md, sizeof(double) * 6 * I.npad);
+        if (I.d == 3 && c->mixed) ok = ok && dalloc(c, (void**)&S.prim, sizeof(float) * (2 * I.N + 7) * n);
         if (I.d == 3) {
             long long ne = (long long)(I.n[0] + 12) * (I.n[1] + 12) * (I.n[2] + 12);
             ok = ok && dalloc(c, (void**)&S.D3, sizeof(double) * 9 * ne);
@@ -986,6 +992,7 @@ es_status es_rhs(es_ctx* c, const double* JU, const double* J, const double* x, 
     P.x = x;
     P.xdot = xdot ? xdot : c->hS[0].zeros;
     P.M = c->hS[0].M;
+    P.prim = c->hS[0].prim;
     P.accU = dJU;
     P.accJ = dJ;
     launch_residual(c, P, nullptr, false, 0.0, 1.0, (cudaStream_t)stream);
@@ -1224,6 +1231,8 @@ es_status es_autotune(es_ctx* c, const double* JU, const double* J, const double
     // the metrics of the state into the context's scratch; the timed flux launches write
     // only the scratch accumulators (MODE_WRITE), so no caller buffer changes
     launch_metrics(c, P, tab, st);
+    if (c->d == 3 && c->mixed)
+        launch_prim3d(c->N, node_grid(c, c->n_cell), st, c->dI, P, tab, c->w_cell, c->n_cell, c->status);
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);

@@ -112,6 +112,7 @@ struct StagePtrs {
     const double* xdot;
     double* M;                // padded metrics target
     double* Md;               // 2D: padded metrics of the mesh velocity (stage k: M + s_k dt Md)
+    float* prim;              // 3D mixed form: binary32 node fields of the stage input (prim3d_kernel)
     double* accU;             // residual accumulators: n_c fields and J
     double* accJ;
     const double* JU0;        // RK base state q^n
@@ -133,6 +134,7 @@ struct Scratch {
     double* D3;               // 3D: products delta_b[x_p] x_q on the grid with 6 ghost layers
     double* XE;               // 3D: x on the grid with 9 ghost layers (boundary maps applied once)
     double* M3;               // 3D moving mesh: padded metrics of the third RK stage's mesh
+    float* prim;              // 3D mixed form: node fields of a stage, field-major on the nodes
     double* Xm;               // 3D: the positions the spatial rows of M were formed from (NaN before)
     double* accU;
     double* accJ;

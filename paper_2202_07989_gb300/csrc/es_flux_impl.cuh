@@ -119,6 +119,7 @@ __global__ void __launch_bounds__(FLUX_TPB, (sizeof(R) == 4 ? (D == 3 ? 4 : 3) :
     using Y = Lay<D, NS>;
     using TL = Tile<S_, WT_>;
     constexpr int NC = Y::NC, NN = TL::NN, NI = TL::NI, NF = Y::NF, NP = TL::NP;
+    constexpr bool PRIM = D == 3 && std::is_same<R, float>::value;
     static_assert(NP < 4096 && 3 * S_ + 6 <= 512, "div_small");
     const int S = S_ > 0 ? S_ : L.S, WT = S_ > 0 ? WT_ : L.WT, NPL = 3 * S + 6;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -171,26 +172,43 @@ __global__ void __launch_bounds__(FLUX_TPB, (sizeof(R) == 4 ? (D == 3 ? 4 : 3) :
             idx[k] = g;
             idx[adim] = a;
             if (bdim < D) idx[bdim] = tb;
-            // the conserved point state from the staged JU, J; the boundary map of direction k
-            // negates the normal momentum (reflect) or gives the fixed state (inflow)
-            R U[MAXC];
+            // the node's fields, from the conserved point state of the staged or loaded JU, J; the
+            // boundary map of direction k negates the normal momentum (reflect) or gives the fixed
+            // state (inflow).  The 3D mixed form reads the fields that prim3d_kernel formed
             const long long pid = plin(I, idx[0], idx[1], idx[2]);
             {
                 int gi, side;
                 const int tmap = map_line(I, k, g, gi, side);
+                R U[MAXC];
                 if (tmap == 2) {
                     for (int q = 0; q < NC; ++q) U[q] = to_r<R>(I.inflow[k][side][q]);
+                    node_fields<D, NS, R>(I, U, nr, NN, node, L.status);
                 } else {
                     int src[3] = { idx[0], idx[1], idx[2] };
                     src[k] = gi;
                     const long long id = staged ? 0 : lin(I, src[0], src[1], src[2]);
+                    if constexpr (PRIM) {
+                        float f[Y::MR];
+#pragma unroll
+                        for (int q = 0; q < Y::MR; ++q) f[q] = P.prim[q * ncell + id];
+                        // a reflection negates the normal velocity and its entropy variable
+#pragma unroll
+                        for (int q = 0; q < D; ++q)
+                            if (tmap == 1 && q == k) {
+                                f[Y::V + q] = -f[Y::V + q];
+                                f[Y::VV + NS + q] = -f[Y::VV + NS + q];
+                            }
+#pragma unroll
+                        for (int q = 0; q < Y::MR; ++q) nr[q * NN + node] = f[q];
+                    } else {
                     const R inv = Ar<R>::rcp(to_r<R>(staged ? stg[NC * NN + node] : P.J[id]));
 #pragma unroll
                     for (int q = 0; q < NC; ++q) U[q] = mulr(to_r<R>(staged ? stg[q * NN + node] : P.JU[q * ncell + id]), inv);
                     if (tmap == 1) U[NS + k] = -U[NS + k];
+                    node_fields<D, NS, R>(I, U, nr, NN, node, L.status);
+                    }
                 }
             }
-            node_fields<D, NS, R>(I, U, nr, NN, node, L.status);
             // metrics of direction k at this node from the metrics kernel (padded buffer covering
             // g in [-3, n + 3))
             {

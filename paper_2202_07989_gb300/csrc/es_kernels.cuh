@@ -93,6 +93,13 @@ __global__ void logmean_small_check_kernel(const float* a, const float* b, const
                                            float* general);
 __global__ void init_J_kernel(const Inst* insts, StagePtrs single, const StagePtrs* table, const int2* work, int nwork);
 
+// 3D mixed form: the flux kernels' node fields of the stage input P.JU, P.J into P.prim, once per
+// node; each direction's launch reads them
+void launch_prim3d(int N, int grid, cudaStream_t st, const Inst* insts, const StagePtrs& single, const StagePtrs* table,
+                   const int2* work, int nwork, int* status);
+template <int NS>
+__host__ __device__ constexpr int prim_fields() { return NS + 3 + NS + 4; }     // densities, velocity, entropy variables
+
 // flux + divergence (+ RK stage) for one direction; D dims, NS species, R compute type,
 // WK the reconstruction of the dissipation (0 WENO-MR, 1 WENO-JS), tile shape index `shape`
 template <int D, int NS, typename R, int WK>
