@@ -65,8 +65,8 @@ enum { ES_SIG_RHO = 0, ES_SIG_RHO1 = 1, ES_SIG_RHO2 = 2, ES_SIG_P = 3, ES_SIG_Y2
  * weights alpha[], nf filter passes and mu Jacobi sweeps (Sec. 4).
  * precision: ES_FP64 runs everything in FP64; ES_MIXED runs the EC pairs, the
  * WENO-MR dissipation and the monitor/filter in FP32 and keeps metrics, the
- * GCL flux of J, the small-jump logarithmic-mean branch, divergence and RK
- * accumulation and the entropy diagnostics in FP64. */
+ * GCL flux of J, divergence and RK accumulation and the entropy diagnostics in
+ * FP64; the small-jump logarithmic mean is formed exactly and rounded once. */
 typedef struct es_config {
     int d;                   /* 2 or 3 */
     int N;                   /* 1 or 2 species */
@@ -316,20 +316,20 @@ es_status es_profile_read(es_ctx* ctx, double* ms, long long* launches, int n_cl
  * exactly.  in, out32, out64: DEVICE arrays of n elements. */
 es_status es_check_conversions(const double* in, int n, float* out32, double* out64, void* stream);
 
-/* Self-check of the exact mean {a} = a/2 + b/2 that the mixed form's log-mean
- * small-jump branch (Sec. 3.3, the Ismail-Roe series) assembles with integer
- * instructions: out[i] = a[i]/2 + b[i]/2 as a binary64 value.  Exact for
+/* Self-check of the exact mean {a} = a/2 + b/2 that the general path of the mixed
+ * form's log-mean small-jump branch (Sec. 3.3, the Ismail-Roe series) assembles with
+ * integer instructions: out[i] = a[i]/2 + b[i]/2 as a binary64 value.  Exact for
  * positive normal a, b whose binary32 exponents differ by at most 7 (the branch
  * has |b - a| < (a + b)/10); otherwise the binary64 sum of the binary32 halves.
  * a, b: DEVICE arrays of n binary32 values; out: DEVICE array of n doubles. */
 es_status es_check_half_sums(const float* a, const float* b, int n, double* out, void* stream);
 
 /* Self-check of the mixed form's log-mean small-jump value {a}(1 - del) rounded to
- * binary32 (Sec. 3.3): fast[i] as the flux kernels form it (integer-built {a},
- * conversions without special cases where their preconditions hold) and
- * general[i] by the general conversions with an FP64 add for {a}; both through
- * one FP64 fused multiply-add.  a, b > 0, 0 <= del <= 1/2.  a, b, del, fast,
- * general: DEVICE arrays of n binary32 values. */
+ * binary32 (Sec. 3.3): fast[i] as the flux kernels form it (exact binary32 pair
+ * arithmetic with one final rounding, where its preconditions hold) and general[i]
+ * by the general conversions with an FP64 add for {a} and one FP64 fused multiply-add.
+ * a, b > 0, 0 <= del <= 1/2.  a, b, del, fast, general: DEVICE arrays of n binary32
+ * values. */
 es_status es_check_logmean_small(const float* a, const float* b, const float* del, int n, float* fast, float* general,
                                  void* stream);
 
