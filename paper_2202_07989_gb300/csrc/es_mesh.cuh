@@ -131,8 +131,9 @@ size_t jacobi_fused2d_smem(int H, int F, int shape);
 // one launch of several: the displacement buffer it starts from (0: y = 0, 1: xa, 2: xb) and ends
 // in, whether it stores Theta for the next one, and whether it is the last (limiter bounds).
 // edges: at the grid's first and last nodes the passes keep the order of operations in which a step
-// beyond one launch (more than 8 sweeps or 4 filter passes) has always rounded them (a filter row summed left to right, the - spacing
-// across a periodic edge from the shifted position) instead of the inner nodes' order
+// beyond one launch (more than 8 sweeps or 4 filter passes) has always rounded them (a filter row
+// summed left to right, the - spacing across a periodic edge from the shifted position) instead of
+// the inner nodes' order
 struct JfPass {
     int src, dst, store_theta, last, edges;
 };
