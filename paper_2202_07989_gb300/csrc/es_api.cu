@@ -9,6 +9,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <functional>
 #include <string>
 #include <vector>
 
@@ -232,19 +233,37 @@ Inst make_inst(const es_config& g)
     return I;
 }
 
-template <typename F>
-int2* build_work(es_ctx* c, F count, int& n)
+// a work list to build: the items of an instance, and where the list and its length go
+struct WorkList {
+    std::function<long long(const Inst&)> count;
+    int2** w;
+    int* n;
+};
+
+// The work lists (instance, item) of a context in one device block, with one allocation and one
+// transfer: a 2D mixed context has 28 lists, and with one of each per list a 64^2 one took 350 us to
+// create, with one block 195.
+bool build_work(es_ctx* c, const std::vector<WorkList>& lists)
 {
-    std::vector<int2> w;
-    for (int i = 0; i < c->n_inst; ++i) {
-        long long t = count(c->hI[i]);
-        for (long long j = 0; j < t; ++j) w.push_back(make_int2(i, (int)j));
+    size_t total = 0;
+    for (const WorkList& l : lists) {
+        long long t = 0;
+        for (const Inst& I : c->hI) t += l.count(I);
+        *l.n = (int)t;
+        total += (size_t)t;
     }
-    n = (int)w.size();
+    std::vector<int2> h(total > 0 ? total : 1);
     int2* d = nullptr;
-    if (!dalloc(c, (void**)&d, sizeof(int2) * (w.empty() ? 1 : w.size()))) return nullptr;
-    if (!w.empty()) cudaMemcpy(d, w.data(), sizeof(int2) * w.size(), cudaMemcpyHostToDevice);
-    return d;
+    if (!dalloc(c, (void**)&d, sizeof(int2) * h.size())) return false;
+    size_t at = 0;
+    for (const WorkList& l : lists) {
+        *l.w = d + at;
+        for (int i = 0; i < c->n_inst; ++i) {
+            const long long t = l.count(c->hI[i]);
+            for (long long j = 0; j < t; ++j) h[at++] = make_int2(i, (int)j);
+        }
+    }
+    return cudaMemcpy(d, h.data(), sizeof(int2) * h.size(), cudaMemcpyHostToDevice) == cudaSuccess;
 }
 
 template <int D, int NS>
@@ -393,26 +412,41 @@ double tile_cost_3d(bool mixed, int k, int s, int w)
     return k == 0 || w >= 8 ? t : t * (w >= 4 ? 1.05 : 1.37);
 }
 
-// time of all tiles of S x WT along direction k, dealt over the grid's CTAs
+// time of all tiles of S x WT along direction k, dealt over the grid's CTAs.  The mean per CTA where
+// there are many waves (from the counts of full and partial tiles), else the longest of the CTAs:
+// dealing the tiles of every candidate out one by one made a 256^3 FP64 context take 24 ms to create,
+// this 2.6 (mixed 7.1 and 2.4)
 double tiles_cost_3d(const es_ctx* c, int k, int S, int WT, int slots)
 {
     const int grid = c->n_inst == 1 ? spread_grid(slots, (c->hI[0].n[k] + S - 1) / S) : slots;
-    std::vector<double> load(grid, 0.0);
-    double sum = 0.0, top = 0.0;
-    long long t = 0;
+    long long tiles = 0;
+    double sum = 0.0;
     for (const Inst& I : c->hI) {
-        const int na = I.n[k == 0 ? 1 : 0], nb = I.n[k == 2 ? 1 : 2];
+        const int n = I.n[k], na = I.n[k == 0 ? 1 : 0], nb = I.n[k == 2 ? 1 : 2];
+        for (int ps = 0; ps < 2; ++ps)
+            for (int pw = 0; pw < 2; ++pw) {
+                const long long m = (long long)(ps ? n % S > 0 : n / S) * (pw ? na % WT > 0 : na / WT) * nb;
+                if (m == 0) continue;
+                tiles += m;
+                sum += (double)m * tile_cost_3d(c->mixed, k, ps ? n % S : S, pw ? na % WT : WT);
+            }
+    }
+    if (tiles > 8LL * grid) return sum / grid;
+    std::vector<double> load(grid, 0.0);
+    int t = 0;
+    for (const Inst& I : c->hI) {
+        const int n = I.n[k], na = I.n[k == 0 ? 1 : 0], nb = I.n[k == 2 ? 1 : 2];
+        double w[2][2];
+        for (int ps = 0; ps < 2; ++ps)
+            for (int pw = 0; pw < 2; ++pw) w[ps][pw] = tile_cost_3d(c->mixed, k, ps ? n % S : S, pw ? na % WT : WT);
         for (int b = 0; b < nb; ++b)
             for (int a = 0; a < na; a += WT)
-                for (int q = 0; q < I.n[k]; q += S, ++t) {
-                    const double w = tile_cost_3d(c->mixed, k, std::min(S, I.n[k] - q), std::min(WT, na - a));
-                    sum += w;
-                    double& l = load[t % grid];
-                    l += w;
-                    top = std::max(top, l);
+                for (int q = 0; q < n; q += S) {
+                    load[t] += w[q + S > n][a + WT > na];
+                    if (++t == grid) t = 0;
                 }
     }
-    return t > 8LL * grid ? sum / grid : top;     // many waves: the mean
+    return *std::max_element(load.begin(), load.end());
 }
 
 // The 3D flux tile of direction k for a context that nobody tuned.  Mixed form: the shape of the
@@ -868,37 +902,6 @@ es_status es_create_batch(const es_config* cfgs, int n_inst, es_ctx** out)
     cudaMemcpy(c->dS, c->hS.data(), sizeof(Scratch) * n_inst, cudaMemcpyHostToDevice);
     cudaMemset(c->status, 0, sizeof(int));
     cudaMemset(c->mflag, 0, sizeof(int) * 5);
-    c->w_pad = build_work(c, [](const Inst& I) { return (long long)node_tiles(I, 3); }, c->n_pad);
-    c->w_cell = build_work(c, [](const Inst& I) { return (long long)node_tiles(I, 0); }, c->n_cell);
-    if (c->d == 3) c->w_ext = build_work(c, [](const Inst& I) { return (long long)node_tiles(I, 6); }, c->n_ext);
-    if (c->d == 3) c->w_col = build_work(c, [](const Inst& I) { return (long long)col3_items(I); }, c->n_col);
-    if (c->d == 3 && !c->mixed) c->w_xe = build_work(c, [](const Inst& I) { return (long long)node_tiles(I, 9); }, c->n_xe);
-    for (int k = 0; k < c->d; ++k)
-        for (int sh = 0; sh < NSHAPE; ++sh) {
-            c->w_flux[k][sh] = build_work(c, [k, sh](const Inst& I) { return flux_tiles(I, k, SHAPE_S[sh], SHAPE_WT[sh]); },
-                                          c->n_flux[k][sh]);
-            ok = ok && c->w_flux[k][sh];
-        }
-    if (c->d == 2)
-        for (int sh = 0; sh < NFSHAPE_ALL; ++sh) {
-            c->w_fused[sh] = build_work(c, [sh](const Inst& I) { return fused_tiles(I, sh); }, c->n_fused[sh]);
-            ok = ok && c->w_fused[sh];
-        }
-    if (c->d == 2 && c->mixed)
-        for (int sh = 0; sh < NJF_SHAPE_ALL; ++sh) {
-            c->w_jf[sh] = build_work(c, [sh](const Inst& I) {
-                return (long long)((I.n[0] + JF_SHAPES[sh][0] - 1) / JF_SHAPES[sh][0]) *
-                       ((I.n[1] + JF_SHAPES[sh][1] - 1) / JF_SHAPES[sh][1]);
-            }, c->n_jf[sh]);
-            ok = ok && c->w_jf[sh];
-        }
-    if (c->d == 2 && c->mixed) pick_mesh_tiles(c);
-    // per-instance ranges of the cell work list (entropy reduction)
-    std::vector<int> first(n_inst + 1, 0);
-    for (int i = 0; i < n_inst; ++i) first[i + 1] = first[i] + c->hI[i].ntile_nodes;
-    ok = ok && dalloc(c, (void**)&c->d_first_cell, sizeof(int) * (n_inst + 1)) &&
-         dalloc(c, (void**)&c->partial, sizeof(double) * 2 * (first[n_inst] > 0 ? first[n_inst] : 1));
-    if (ok) cudaMemcpy(c->d_first_cell, first.data(), sizeof(int) * (n_inst + 1), cudaMemcpyHostToDevice);
     if (c->d == 2 && c->N == 1) prepare_all<2, 1>(c->weno);
     else if (c->d == 2 && c->N == 2) prepare_all<2, 2>(c->weno);
     else if (c->d == 3 && c->N == 1) prepare_all<3, 1>(c->weno);
@@ -908,14 +911,37 @@ es_status es_create_batch(const es_config* cfgs, int n_inst, es_ctx** out)
         c->flux_grid[k] = c->sms * flux_occ(c, c->flux_shape[k]);
         if (c->d != 3) continue;
         pick_tiles_3d(c, k, c->flux_grid[k]);
-        if (c->mixed) {
-            c->flux_grid[k] = c->sms * flux_occ(c, c->flux_shape[k]);
-            continue;
-        }
-        const int S = c->fit_S[k], WT = c->fit_WT[k];
-        c->w_flux[k][NSHAPE] = build_work(c, [k, S, WT](const Inst& I) { return flux_tiles(I, k, S, WT); }, c->n_flux[k][NSHAPE]);
-        ok = ok && c->w_flux[k][NSHAPE];
+        if (c->mixed) c->flux_grid[k] = c->sms * flux_occ(c, c->flux_shape[k]);
     }
+    std::vector<WorkList> lists = { { [](const Inst& I) { return (long long)node_tiles(I, 3); }, &c->w_pad, &c->n_pad },
+                                    { [](const Inst& I) { return (long long)node_tiles(I, 0); }, &c->w_cell, &c->n_cell } };
+    if (c->d == 3) {
+        lists.push_back({ [](const Inst& I) { return (long long)node_tiles(I, 6); }, &c->w_ext, &c->n_ext });
+        lists.push_back({ [](const Inst& I) { return (long long)col3_items(I); }, &c->w_col, &c->n_col });
+        if (!c->mixed) lists.push_back({ [](const Inst& I) { return (long long)node_tiles(I, 9); }, &c->w_xe, &c->n_xe });
+    }
+    for (int k = 0; k < c->d; ++k)
+        for (int sh = 0; sh < NSHAPE + (c->fit_S[k] > 0); ++sh) {
+            const int S = shape_S(c, k, sh), WT = shape_WT(c, k, sh);
+            lists.push_back({ [k, S, WT](const Inst& I) { return flux_tiles(I, k, S, WT); }, &c->w_flux[k][sh], &c->n_flux[k][sh] });
+        }
+    if (c->d == 2)
+        for (int sh = 0; sh < (c->mixed ? NFSHAPE_MIXED : NFSHAPE_ALL); ++sh)
+            lists.push_back({ [sh](const Inst& I) { return fused_tiles(I, sh); }, &c->w_fused[sh], &c->n_fused[sh] });
+    if (c->d == 2 && c->mixed)
+        for (int sh = 0; sh < NJF_SHAPE_ALL; ++sh)
+            lists.push_back({ [sh](const Inst& I) {
+                return (long long)((I.n[0] + JF_SHAPES[sh][0] - 1) / JF_SHAPES[sh][0]) *
+                       ((I.n[1] + JF_SHAPES[sh][1] - 1) / JF_SHAPES[sh][1]);
+            }, &c->w_jf[sh], &c->n_jf[sh] });
+    ok = build_work(c, lists);
+    if (c->d == 2 && c->mixed) pick_mesh_tiles(c);
+    // per-instance ranges of the cell work list (entropy reduction)
+    std::vector<int> first(n_inst + 1, 0);
+    for (int i = 0; i < n_inst; ++i) first[i + 1] = first[i] + c->hI[i].ntile_nodes;
+    ok = ok && dalloc(c, (void**)&c->d_first_cell, sizeof(int) * (n_inst + 1)) &&
+         dalloc(c, (void**)&c->partial, sizeof(double) * 2 * (first[n_inst] > 0 ? first[n_inst] : 1));
+    if (ok) cudaMemcpy(c->d_first_cell, first.data(), sizeof(int) * (n_inst + 1), cudaMemcpyHostToDevice);
     // 2D contexts start with the fused stage launch in fused shape 0 (es_autotune may change it)
     if (c->d == 2) {
         c->fused_shape = 0;
@@ -923,7 +949,7 @@ es_status es_create_batch(const es_config* cfgs, int n_inst, es_ctx** out)
         pick_fused(c);
     }
     cudaError_t e = cudaDeviceSynchronize();
-    if (!ok || e != cudaSuccess || !c->w_pad || !c->w_cell || (c->d == 3 && (!c->w_ext || !c->w_col || (!c->mixed && !c->w_xe)))) {
+    if (!ok || e != cudaSuccess) {
         fprintf(stderr, "es_create: setup failed: %s\n", cudaGetErrorString(e));
         es_destroy(c);
         return ES_ERR_CUDA;

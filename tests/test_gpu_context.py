@@ -1,0 +1,36 @@
+"""Contexts: what creating one costs, the scratch it holds, and the launch configuration it
+reports, takes and runs."""
+import time
+
+import pytest
+
+from paper_2202_07989_gb300 import workloads as W
+
+from .helpers import case, need_gpu, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+def _ctx(pb, precision=0):
+    from paper_2202_07989_gb300 import es
+    return es.Context(pb, precision)
+
+
+def _create_ms(pb, form, torch):
+    best = float("inf")
+    for _ in range(5):
+        t = time.perf_counter()
+        ctx = _ctx(pb, form)
+        torch.cuda.synchronize()
+        best = min(best, time.perf_counter() - t)
+        del ctx
+    return 1e3 * best
+
+
+def test_fp64_context_creation_time():
+    """An FP64 3D context, which picks its flux tiles among all extents, is created in at most
+    twice the time of a mixed one (about 2.5 ms each at 256^3, nearly all of it allocations)."""
+    torch = need_gpu()
+    pb = W.random_problem(3, 2, (256, 256, 256))
+    fp64, mixed = _create_ms(pb, 0, torch), _create_ms(pb, 1, torch)
+    assert fp64 <= 2.0 * mixed, (fp64, mixed)
