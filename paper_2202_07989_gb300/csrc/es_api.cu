@@ -856,10 +856,13 @@ es_status es_create_batch(const es_config* cfgs, int n_inst, es_ctx** out)
         long long n = I.ncell;
         ok = ok && dalloc(c, (void**)&S.M, sizeof(double) * I.d * (I.d + 1) * I.npad);
         if (I.d == 2) ok = ok && dalloc(c, (void**)&S.Md, sizeof(double) * 6 * I.npad);
-        if (I.d == 3 && c->mixed) ok = ok && dalloc(c, (void**)&S.prim, sizeof(float) * (2 * I.N + 7) * n);
         if (I.d == 3) {
             long long ne = (long long)(I.n[0] + 12) * (I.n[1] + 12) * (I.n[2] + 12);
             ok = ok && dalloc(c, (void**)&S.D3, sizeof(double) * 9 * ne);
+            // the node fields of a stage (36 or 44 bytes a node) use the products' 72 bytes: a metrics
+            // pass forms and reads the products before the stage's fields are written, and forms
+            // them again before it next reads them
+            if (c->mixed) S.prim = reinterpret_cast<float*>(S.D3);
             const long long nx = (long long)(I.n[0] + 18) * (I.n[1] + 18) * (I.n[2] + 18);
             ok = ok && dalloc(c, (void**)&S.XE, sizeof(double) * 3 * nx);
             if (!I.fixed) ok = ok && dalloc(c, (void**)&S.M3, sizeof(double) * 12 * I.npad);

@@ -134,7 +134,7 @@ struct Scratch {
     double* D3;               // 3D: products delta_b[x_p] x_q on the grid with 6 ghost layers
     double* XE;               // 3D: x on the grid with 9 ghost layers (boundary maps applied once)
     double* M3;               // 3D moving mesh: padded metrics of the third RK stage's mesh
-    float* prim;              // 3D mixed form: node fields of a stage, field-major on the nodes
+    float* prim;              // 3D mixed form: node fields of a stage, field-major on the nodes (in D3)
     double* Xm;               // 3D: the positions the spatial rows of M were formed from (NaN before)
     double* accU;
     double* accJ;

@@ -34,3 +34,13 @@ def test_fp64_context_creation_time():
     pb = W.random_problem(3, 2, (256, 256, 256))
     fp64, mixed = _create_ms(pb, 0, torch), _create_ms(pb, 1, torch)
     assert fp64 <= 2.0 * mixed, (fp64, mixed)
+
+
+@pytest.mark.parametrize("N", [1, 2])
+def test_mixed_3d_scratch(N):
+    """A mixed 3D context holds no more than the FP64 one and its nine binary32 edge spacings a node
+    (36 bytes, and those of one more layer of nodes)."""
+    need_gpu()
+    pb = W.random_problem(3, N, (64, 64, 64))
+    fp64, mixed = _ctx(pb, 0).scratch_bytes, _ctx(pb, 1).scratch_bytes
+    assert mixed - fp64 <= 36 * 65 ** 3, (mixed - fp64) / pb.ncell
