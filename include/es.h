@@ -303,7 +303,8 @@ es_status es_run_host(es_ctx* ctx, double* JU, double* J, double* x, int steps, 
  * synchronises, returns per class the summed milliseconds and the launch
  * count since the last read, then resets them.  Classes (n_classes <= 8):
  * 0..2 flux + divergence (+ RK stage) for directions 1..3 (per-direction
- * launches; class 0 counts the 3D mixed form's node-field pass too), 3 metrics, 4 mesh redistribution (CFL, monitor, filter, Jacobi,
+ * launches; in the 3D mixed form class 0 times the node-field pass and the launch of
+ * direction 1 as one), 3 metrics, 4 mesh redistribution (CFL, monitor, filter, Jacobi,
  * limiter, xdot), 5 entropy diagnostics, 6 the fused 2D stage launch (both
  * directions, + RK stage).  es_profile(ctx, 0) frees the events. */
 es_status es_profile(es_ctx* ctx, int enable);

@@ -601,10 +601,6 @@ void launch_residual(es_ctx* c, const StagePtrs& P, const StagePtrs* tab, bool r
         flux2d_launch(c, L, sh, c->fused_run >= 0 ? c->fused_run_grid : c->fused_grid, st);
         return;
     }
-    if (c->d == 3 && c->mixed) {
-        ProfScope ps(c, PC_FLUX, st);
-        launch_prim3d(c->N, node_grid(c, c->n_cell), st, c->dI, P, tab, c->w_cell, c->n_cell, c->status);
-    }
     for (int k = 0; k < c->d; ++k) {
         FluxLaunch L;
         L.insts = c->dI;
@@ -624,6 +620,9 @@ void launch_residual(es_ctx* c, const StagePtrs& P, const StagePtrs* tab, bool r
         L.xc = xc;
         L.status = c->status;
         ProfScope ps(c, PC_FLUX + k, st);
+        // (one event pair with direction 1: a class counts one launch per stage)
+        if (k == 0 && c->d == 3 && c->mixed)
+            launch_prim3d(c->N, node_grid(c, c->n_cell), st, c->dI, P, tab, c->w_cell, c->n_cell, c->status);
         flux_launch(c, L, sh, c->flux_grid[k], st);
     }
 }

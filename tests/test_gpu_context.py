@@ -44,3 +44,18 @@ def test_mixed_3d_scratch(N):
     pb = W.random_problem(3, N, (64, 64, 64))
     fp64, mixed = _ctx(pb, 0).scratch_bytes, _ctx(pb, 1).scratch_bytes
     assert mixed - fp64 <= 36 * 65 ** 3, (mixed - fp64) / pb.ncell
+
+
+@pytest.mark.parametrize("form", [0, 1])
+def test_profile_counts_one_launch_per_direction(form):
+    """Every flux class counts one launch per residual (in the 3D mixed form too, where the
+    node-field pass precedes direction 1), so that time / launches is a launch's time."""
+    torch = need_gpu()
+    pb, JU, J, x, xdot = case(3, 2, (20, 12, 11), "periodic", seed=5)
+    ctx = _ctx(pb, form)
+    G = [to_dev(t, torch) for t in (JU, J, x, xdot)]
+    ctx.es_profile(True)
+    ctx.es_rhs(*G)
+    prof = ctx.es_profile_read()
+    ctx.es_profile(False)
+    assert [prof["flux_k%d" % k][1] for k in (1, 2, 3)] == [1, 1, 1]
