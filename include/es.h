@@ -187,7 +187,10 @@ es_status es_autotune(es_ctx* ctx, const double* JU, const double* J, const doub
 es_status es_get_tuning(const es_ctx* ctx, int* shape, int* S, int* WT, int* grid, float* ms);
 
 /* Fix the flux launch of direction k to tile shape `shape` (0..5) and `grid`
- * CTAs (0 = SM count x occupancy of that shape).  ES_ERR_ARG when out of range. */
+ * CTAs (0 = the library's choice, reported by es_get_tuning: SM count x occupancy
+ * of that shape; on a single 3D instance whose lines end in a partial segment the
+ * next lower count that shares no factor with the segments per line).
+ * ES_ERR_ARG when out of range. */
 es_status es_set_tuning(es_ctx* ctx, int k, int shape, int grid);
 
 /* Fused 2D stage launch (the paper has no counterpart; a launch schedule): both

@@ -289,12 +289,17 @@ void prepare_all(int weno)
 
 int gcd_(int a, int b) { return b == 0 ? a : gcd_(b, a % b); }
 
-// The largest grid up to `grid` CTAs that shares no factor with the segments per line (ns): tiles
-// are numbered segment by segment, so with a common factor the same CTAs would get every line's
-// last, partial segment and the others only full ones (direction 1 of 63^3 in the FP64 form, 62 x 4
-// tiles: 1737 us with 152 CTAs, 1126 us with the partial tiles spread)
-int spread_grid(int grid, int ns)
+// The CTAs of a flux launch along direction k in tiles of S nodes, where the library chooses them:
+// `slots`, or, where a single 3D instance's lines end in a partial segment and there are more tiles
+// than slots, the largest count below that shares no factor with the segments per line.  Tiles are
+// numbered segment by segment, so with a common factor the same CTAs would get every line's partial
+// segment and the others only full ones (direction 1 of 63^3 in the FP64 form, 62 x 4 tiles: 1737 us
+// with 152 CTAs, 1126 us with 151)
+int auto_grid(const es_ctx* c, int k, int S, long long tiles, int slots)
 {
+    if (c->d != 3 || c->n_inst != 1 || c->hI[0].n[k] % S == 0 || tiles <= slots) return slots;
+    const int ns = (c->hI[0].n[k] + S - 1) / S;
+    int grid = slots;
     while (grid > 1 && gcd_(grid, ns) != 1) --grid;
     return grid;
 }
@@ -303,7 +308,6 @@ int spread_grid(int grid, int ns)
 void flux_launch(es_ctx* c, const FluxLaunch& L, int shape, int grid, cudaStream_t st)
 {
     if (grid > L.nwork) grid = L.nwork;
-    else if (c->d == 3 && c->n_inst == 1) grid = spread_grid(grid, (c->hI[0].n[L.k] + L.S - 1) / L.S);
     if (grid <= 0) return;
 #define FD(d, n)                                                                                      \
     do {                                                                                              \
@@ -393,6 +397,12 @@ int flux_occ(es_ctx* c, int shape)
 #undef FO
 }
 
+// the library's CTA count of direction k in tile shape sh, `per_sm` CTAs per SM (0: as many as fit)
+int shape_grid(es_ctx* c, int k, int sh, int per_sm = 0)
+{
+    return auto_grid(c, k, shape_S(c, k, sh), c->n_flux[k][sh], c->sms * (per_sm > 0 ? per_sm : flux_occ(c, sh)));
+}
+
 // The time of a 3D flux tile of s nodes along the line x w lines, in arbitrary units.
 // Mixed form: a fixed part (a tile's phases wait on one another and on their loads), one unit per
 // round of nodes over the 256 threads and 0.4 per warp of pairs; loads across the contiguous
@@ -418,7 +428,6 @@ double tile_cost_3d(bool mixed, int k, int s, int w)
 // this 2.6 (mixed 7.1 and 2.4)
 double tiles_cost_3d(const es_ctx* c, int k, int S, int WT, int slots)
 {
-    const int grid = c->n_inst == 1 ? spread_grid(slots, (c->hI[0].n[k] + S - 1) / S) : slots;
     long long tiles = 0;
     double sum = 0.0;
     for (const Inst& I : c->hI) {
@@ -431,6 +440,7 @@ double tiles_cost_3d(const es_ctx* c, int k, int S, int WT, int slots)
                 sum += (double)m * tile_cost_3d(c->mixed, k, ps ? n % S : S, pw ? na % WT : WT);
             }
     }
+    const int grid = auto_grid(c, k, S, tiles, slots);
     if (tiles > 8LL * grid) return sum / grid;
     std::vector<double> load(grid, 0.0);
     int t = 0;
@@ -909,12 +919,8 @@ es_status es_create_batch(const es_config* cfgs, int n_inst, es_ctx** out)
     else if (c->d == 3 && c->N == 1) prepare_all<3, 1>(c->weno);
     else prepare_all<3, 2>(c->weno);
     prepare_mesh();
-    for (int k = 0; k < c->d; ++k) {
-        c->flux_grid[k] = c->sms * flux_occ(c, c->flux_shape[k]);
-        if (c->d != 3) continue;
-        pick_tiles_3d(c, k, c->flux_grid[k]);
-        if (c->mixed) c->flux_grid[k] = c->sms * flux_occ(c, c->flux_shape[k]);
-    }
+    if (c->d == 3)
+        for (int k = 0; k < c->d; ++k) pick_tiles_3d(c, k, c->sms * flux_occ(c, c->flux_shape[k]));
     std::vector<WorkList> lists = { { [](const Inst& I) { return (long long)node_tiles(I, 3); }, &c->w_pad, &c->n_pad },
                                     { [](const Inst& I) { return (long long)node_tiles(I, 0); }, &c->w_cell, &c->n_cell } };
     if (c->d == 3) {
@@ -937,6 +943,7 @@ es_status es_create_batch(const es_config* cfgs, int n_inst, es_ctx** out)
                        ((I.n[1] + JF_SHAPES[sh][1] - 1) / JF_SHAPES[sh][1]);
             }, &c->w_jf[sh], &c->n_jf[sh] });
     ok = build_work(c, lists);
+    for (int k = 0; k < c->d; ++k) c->flux_grid[k] = shape_grid(c, k, c->flux_fit[k] ? NSHAPE : c->flux_shape[k]);
     if (c->d == 2 && c->mixed) pick_mesh_tiles(c);
     // per-instance ranges of the cell work list (entropy reduction)
     std::vector<int> first(n_inst + 1, 0);
@@ -1285,7 +1292,7 @@ es_status es_autotune(es_ctx* c, const double* JU, const double* J, const double
                 L.mcoef = 0.0;
                 L.xc = 0.0;
                 L.status = c->status;
-                const int grid = c->sms * o;
+                const int grid = shape_grid(c, k, sh, o);
                 flux_launch(c, L, sh, grid, st);
                 cudaEventRecord(e0, st);
                 for (int r = 0; r < reps; ++r) flux_launch(c, L, sh, grid, st);
@@ -1436,7 +1443,7 @@ es_status es_set_tuning(es_ctx* c, int k, int shape, int grid)
         return fail(c, ES_ERR_ARG, "es_set_tuning: direction, shape or grid out of range");
     c->flux_shape[k] = shape;
     c->flux_fit[k] = false;
-    c->flux_grid[k] = grid > 0 ? grid : c->sms * flux_occ(c, shape);
+    c->flux_grid[k] = grid > 0 ? grid : shape_grid(c, k, shape);
     c->flux_ms[k] = 0.f;
     drop_run_graph(c);
     return ES_OK;
