@@ -339,13 +339,14 @@ def tune(runner, batched=False):
         t = runner.ctx.es_autotune()
     else:
         t = runner.ctx.es_autotune(runner.JU, runner.J, runner.x, runner.xdot)
-    out = ["%dx%d tile, %d CTAs, %.3f ms" % (S, WT, grid, ms) for _, S, WT, grid, ms in t]
+    tiles = runner.ctx.es_get_tiles
+    out = ["%dx%d tile, %d CTAs, %.3f ms" % tiles("flux_k%d" % (k + 1)) for k in range(len(t))]
     if len(t) == 2:
-        sh, TX, TY, grid, ms = runner.ctx.es_get_fusion()
-        out.append("fused %dx%d tile, %d CTAs, %.3f ms" % (TX, TY, grid, ms) if sh >= 0 else "fused off (best %.3f ms)" % ms)
-        sh, TX, TY, thr, ms = runner.ctx.es_get_mesh_tiles()
-        if sh >= 0:
-            out.append("mesh step %dx%d tile, %d threads, %.3f ms" % (TX, TY, thr, ms))
+        TX, TY, grid, ms = tiles("stage")
+        out.append("fused %dx%d tile, %d CTAs, %.3f ms" % (TX, TY, grid, ms) if TX else "fused off (best %.3f ms)" % runner.ctx.es_get_fusion()[4])
+        TX, TY, grid, ms = tiles("mesh")
+        if TX:
+            out.append("mesh step %dx%d tile, %d CTAs, %.3f ms" % (TX, TY, grid, ms))
     return out
 
 

@@ -177,13 +177,13 @@ es_status es_step(es_ctx* ctx, double* JU, double* J, double* x, double dt_fixed
 es_status es_autotune(es_ctx* ctx, const double* JU, const double* J, const double* x, const double* xdot, int reps,
                       void* stream);
 
-/* The flux launch configuration per direction k = 0..2 (zeros for directions
- * the problem lacks): shape index, S, WT, persistent grid size (CTAs) and the
- * time per launch the last es_autotune measured (0 if none).  A 3D context that
- * nobody tuned picks its tiles by its grid; in the FP64 form, and in es_autotune
- * there, they may have an extent of their own: S and WT are then that extent and
- * the shape index the one it replaces.
- * Each argument points to 3 values (HOST). */
+/* The flux tile of the 6 shapes per direction k = 0..2 (zeros for directions the
+ * problem lacks): shape index, S, WT, persistent grid size (CTAs) and the time per
+ * launch the last es_autotune measured for it (0 if none); es_set_tuning with this
+ * shape and grid gives the same launch.  A 3D context that nobody tuned picks its
+ * shapes by its grid.  In the 3D FP64 form the launches may run in tiles of another
+ * extent, chosen by the grid or by es_autotune where it measures them faster:
+ * es_get_tiles reports what runs.  Each argument points to 3 values (HOST). */
 es_status es_get_tuning(const es_ctx* ctx, int* shape, int* S, int* WT, int* grid, float* ms);
 
 /* Fix the flux launch of direction k to tile shape `shape` (0..5) and `grid`
@@ -202,13 +202,14 @@ es_status es_set_tuning(es_ctx* ctx, int k, int shape, int grid);
  * context also times each fused shape and keeps the fused launch when it beats
  * the sum of the best per-direction launches.  A new 2D context starts with the
  * fused launch in shape 0 (16 x 12 tiles, full occupancy).  A new context by its
- * grid, and es_autotune where it measures them faster, run the launch on other
- * tiles behind the reported shape (8 x 8, 12 x 8 or 16 x 8 on grids of few tiles;
- * 16 x 14 or 24 x 15 in the FP64 form); a shape set by es_set_fusion runs as it is.
+ * grid, and es_autotune where it measures them faster, run the launch on tiles beyond
+ * these shapes (8 x 8, 12 x 8 or 16 x 8 on grids of few tiles; 16 x 14 or 24 x 15 in
+ * the FP64 form); a shape set by es_set_fusion runs as it is.
  * es_get_fusion: fused shape index (-1: per-direction launches), TX, TY, grid
  * (CTAs) and the best fused time per launch the last es_autotune measured (0 if
- * none; set even when the per-direction launches won).  All pointers HOST, one
- * value each. */
+ * none; set even when the per-direction launches won) of these shapes;
+ * es_set_fusion with that shape and grid gives that launch.  es_get_tiles reports
+ * the tiles that run.  All pointers HOST, one value each. */
 es_status es_get_fusion(const es_ctx* ctx, int* shape, int* TX, int* TY, int* grid, float* ms);
 
 /* Fix the fused 2D stage launch: shape -1 (per-direction launches) or 0..4, and
@@ -226,15 +227,36 @@ es_status es_set_fusion(es_ctx* ctx, int shape, int grid);
  * es_autotune on such a context also times every shape on one mesh step of the
  * given state and keeps the fastest.  A new context reports shape 0 and runs the
  * tiles that its grid size suggests, smaller ones (16 x 8, 8 x 8) on small grids
- * among them; es_autotune may keep those behind the reported shape too, and a
- * shape set by es_set_mesh_tiles runs as it is.
- * es_get_mesh_tiles: shape index, TX, TY, threads per block and the best time per
- * launch the last es_autotune measured (0 if none).  All pointers HOST, one value
- * each; on contexts without the fused mesh step, shape -1 and zeros.
+ * among them; es_autotune may keep those too, and a shape set by es_set_mesh_tiles
+ * runs as it is.
+ * es_get_mesh_tiles: shape index, TX, TY, threads per block and the best time the
+ * last es_autotune measured among the 4 shapes (0 if none) for the monitor, filter
+ * and sweep launches of one mesh step together.  All pointers HOST, one value each;
+ * on contexts without the fused mesh step, shape -1 and zeros.  es_get_tiles reports
+ * the tiles that run.
  * es_set_mesh_tiles: shape 0..3; ES_ERR_ARG when out of range or when the context
  * is not a mixed-form 2D context. */
 es_status es_get_mesh_tiles(const es_ctx* ctx, int* shape, int* TX, int* TY, int* threads, float* ms);
 es_status es_set_mesh_tiles(es_ctx* ctx, int shape);
+
+/* The tiles that a context's launches run on, by extent, over all tiles the library
+ * has: the shapes above and those beyond them.  launch: the flux launch of direction
+ * 1..3 (a = S nodes along the line, b = WT lines; 2D contexts run it only without the
+ * fused stage launch), the fused 2D stage launch (a = TX, b = TY) or the mixed 2D mesh
+ * step (a = TX, b = TY).  No tile changes a result.
+ * es_get_tiles: the extent, the CTAs and the time the last es_autotune measured for
+ * them (0 if none; mesh step: all its monitor, filter and sweep launches); zeros for a
+ * launch the context does not run.  All pointers HOST, one value each.
+ * es_set_tiles: runs the launch on tiles of that extent and `grid` CTAs (0 = the
+ * library's choice; ignored for the mesh step).  Stage launch: 0 x 0 selects the
+ * per-direction launches.  What es_get_tiles reports on one context can be set on
+ * another of the same dimension, form and grid size, which then runs the same tiles.
+ * In the 3D FP64 form every S and WT <= 16 with (S + 1) WT <= 256 is a flux tile; an
+ * extent that the context has not run yet allocates its work list (kept until the
+ * context is destroyed), so not during stream capture.  ES_ERR_ARG for an extent that the launch has no tile of. */
+enum { ES_TILES_FLUX1 = 0, ES_TILES_FLUX2 = 1, ES_TILES_FLUX3 = 2, ES_TILES_STAGE = 3, ES_TILES_MESH = 4 };
+es_status es_get_tiles(const es_ctx* ctx, int launch, int* a, int* b, int* grid, float* ms);
+es_status es_set_tiles(es_ctx* ctx, int launch, int a, int b, int grid);
 
 /* Schlieren function of Example 5.8, Eq. (schlieren), on one instance:
  * phi = exp(-Psi |grad rho| / max |grad rho|), Psi = (psi1 rho_1 + psi2 rho_2) / rho
@@ -294,8 +316,8 @@ es_status es_step_batch(es_ctx* ctx, void* stream);
  * x = J + cells), else one per buffer and direction (asynchronous when the host
  * memory is pinned).  Each step replays a CUDA graph of es_step on the device
  * buffers, captured on a private stream by the first call and again after
- * es_autotune, es_set_tuning, es_set_fusion, es_set_mesh_tiles or a new
- * dt_fixed; with es_profile on, the steps are launched one kernel at a time
+ * es_autotune, es_set_tuning, es_set_fusion, es_set_mesh_tiles, es_set_tiles or a
+ * new dt_fixed; with es_profile on, the steps are launched one kernel at a time
  * instead.  ES_ERR_ARG during stream capture. */
 es_status es_run_host(es_ctx* ctx, double* JU, double* J, double* x, int steps, double dt_fixed, double* t,
                       void* stream);

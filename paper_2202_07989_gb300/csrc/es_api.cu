@@ -1,7 +1,8 @@
 // C ABI of the library (include/es.h): contexts, argument checks, work lists and
 // the launch sequences of every entry point.  Single-instance calls pass their
 // pointers to the kernels by value; batched calls use per-instance tables
-// uploaded by es_bind_batch.  Nothing here allocates after creation.
+// uploaded by es_bind_batch.  After creation only es_bind_batch, es_run_host and es_set_tiles
+// allocate (their tables, device buffers and the list of an extent of the caller's).
 #include "../../include/es.h"
 #include "es_mesh.cuh"
 
@@ -10,6 +11,7 @@
 #include <cstdio>
 #include <cstring>
 #include <functional>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -34,7 +36,10 @@ struct es_ctx {
     // flux work list per direction and tile shape; the last one (3D) is the extent fitted to the grid
     int2* w_flux[3][NSHAPE + 1] = {};
     int n_flux[3][NSHAPE + 1] = {};
-    int fit_S[3] = { 0, 0, 0 }, fit_WT[3] = { 0, 0, 0 };
+    int fit_S[3] = { 0, 0, 0 }, fit_WT[3] = { 0, 0, 0 }, fit_grid[3] = { 0, 0, 0 };
+    float fit_ms[3] = { 0.f, 0.f, 0.f };
+    struct Fit { int k, S, WT; int2* w; int n; };
+    std::vector<Fit> fits;                 // the lists of all extents fitted or set so far (captured graphs may read them)
     bool flux_fit[3] = { false, false, false };    // the launches use the fitted extent
     int2* w_fused[NFSHAPE_ALL] = {};           // fused 2D stage work list per fused tile shape
     int n_fused[NFSHAPE_ALL] = {};
@@ -42,7 +47,7 @@ struct es_ctx {
     int n_jf[NJF_SHAPE_ALL] = {};
     int jf_shape = JF_SHAPE_DEFAULT;
     int jf_run = -1;                       // the tiles the launch runs on where the library chose others; -1: jf_shape
-    float jf_ms = 0.f;
+    float jf_ms = 0.f, jf_run_ms = 0.f;
     int* d_first_cell = nullptr;
     double* partial = nullptr;
     int* status = nullptr;
@@ -72,6 +77,7 @@ struct es_ctx {
     // the tiles a fused launch runs on, where the library chose others (small grids); -1: fused_shape
     int fused_run = -1;
     int fused_run_grid = 0;
+    float fused_run_ms = 0.f;
     std::string err;
     // kernel timing (es_profile)
     bool prof = false;
@@ -491,6 +497,29 @@ void pick_tiles_3d(es_ctx* c, int k, int slots)
     c->flux_fit[k] = true;
 }
 
+// take S x WT as the extent beyond the table of direction k (3D FP64), with its work list
+bool fit_extent(es_ctx* c, int k, int S, int WT)
+{
+    try {
+        auto f = std::find_if(c->fits.begin(), c->fits.end(),
+                              [=](const es_ctx::Fit& q) { return q.k == k && q.S == S && q.WT == WT; });
+        if (f == c->fits.end()) {
+            es_ctx::Fit q = { k, S, WT, nullptr, 0 };
+            c->fits.reserve(c->fits.size() + 1);
+            if (!build_work(c, { { [k, S, WT](const Inst& I) { return flux_tiles(I, k, S, WT); }, &q.w, &q.n } })) return false;
+            if (cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) return false;     // the list is on the device
+            f = c->fits.insert(c->fits.end(), q);
+        }
+        c->w_flux[k][NSHAPE] = f->w;
+        c->n_flux[k][NSHAPE] = f->n;
+        c->fit_S[k] = S;
+        c->fit_WT[k] = WT;
+    } catch (const std::bad_alloc&) {
+        return false;
+    }
+    return true;
+}
+
 // planes per chunk of the 3D kernels that march along i3: chunks enough for about four
 // waves of 3 CTAs per SM over the instance's columns, at least 4 planes a chunk
 int march_zc(const Inst& I, int sms)
@@ -502,7 +531,7 @@ int march_zc(const Inst& I, int sms)
     return zc >= 4 ? zc : (I.n[2] < 4 ? I.n[2] : 4);
 }
 
-int node_grid(es_ctx* c, int nwork)
+int node_grid(const es_ctx* c, int nwork)
 {
     int cap = c->sms * 8;
     return nwork < cap ? nwork : cap;
@@ -633,7 +662,7 @@ void launch_residual(es_ctx* c, const StagePtrs& P, const StagePtrs* tab, bool r
         // (one event pair with direction 1: a class counts one launch per stage)
         if (k == 0 && c->d == 3 && c->mixed)
             launch_prim3d(c->N, node_grid(c, c->n_cell), st, c->dI, P, tab, c->w_cell, c->n_cell, c->status);
-        flux_launch(c, L, sh, c->flux_grid[k], st);
+        flux_launch(c, L, sh, c->flux_fit[k] ? c->fit_grid[k] : c->flux_grid[k], st);
     }
 }
 
@@ -943,7 +972,12 @@ es_status es_create_batch(const es_config* cfgs, int n_inst, es_ctx** out)
                        ((I.n[1] + JF_SHAPES[sh][1] - 1) / JF_SHAPES[sh][1]);
             }, &c->w_jf[sh], &c->n_jf[sh] });
     ok = build_work(c, lists);
-    for (int k = 0; k < c->d; ++k) c->flux_grid[k] = shape_grid(c, k, c->flux_fit[k] ? NSHAPE : c->flux_shape[k]);
+    for (int k = 0; k < c->d; ++k) {
+        c->flux_grid[k] = shape_grid(c, k, c->flux_shape[k]);
+        if (!c->flux_fit[k]) continue;
+        c->fit_grid[k] = shape_grid(c, k, NSHAPE);
+        c->fits.push_back({ k, c->fit_S[k], c->fit_WT[k], c->w_flux[k][NSHAPE], c->n_flux[k][NSHAPE] });
+    }
     if (c->d == 2 && c->mixed) pick_mesh_tiles(c);
     // per-instance ranges of the cell work list (entropy reduction)
     std::vector<int> first(n_inst + 1, 0);
@@ -1272,8 +1306,8 @@ es_status es_autotune(es_ctx* c, const double* JU, const double* J, const double
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
     for (int k = 0; k < c->d; ++k) {
-        float best = 3.0e38f;
-        c->flux_fit[k] = false;
+        // the best shape of the table, and the extent beyond it (3D FP64), each at its best CTA count
+        float best[2] = { 3.0e38f, 3.0e38f };
         for (int sh = 0; sh < NSHAPE + (c->fit_S[k] > 0); ++sh) {
             const int occ = flux_occ(c, sh);
             for (int o = occ; o >= 1 && o >= occ - 1; --o) {
@@ -1301,25 +1335,28 @@ es_status es_autotune(es_ctx* c, const double* JU, const double* J, const double
                 float ms = 0.f;
                 cudaEventElapsedTime(&ms, e0, e1);
                 ms /= (float)reps;
-                if (ms < best) {
-                    best = ms;
+                float& b = best[sh < NSHAPE ? 0 : 1];
+                if (ms < b) {
+                    b = ms;
                     if (sh < NSHAPE) c->flux_shape[k] = sh;
-                    else c->flux_fit[k] = true;
-                    c->flux_grid[k] = grid;
+                    (sh < NSHAPE ? c->flux_grid : c->fit_grid)[k] = grid;
                 }
             }
         }
-        c->flux_ms[k] = best;
+        c->flux_fit[k] = best[1] < best[0];
+        c->flux_ms[k] = best[0];
+        c->fit_ms[k] = c->flux_fit[k] ? best[1] : 0.f;
     }
     // 2D: the fused stage launch in each fused shape against the sum of the best
     // per-direction launches (both in MODE_WRITE); the faster form is kept
     c->fused_shape = -1;
     c->fused_run = -1;
-    c->fused_ms = 0.f;
+    c->fused_ms = c->fused_run_ms = 0.f;
     drop_run_graph(c);
     if (c->d == 2) {
-        // the shapes beyond the table last: they take over the launch, not the reported shape
-        float best = 3.0e38f;
+        // the best shape of the table and the best beyond it
+        float best[2] = { 3.0e38f, 3.0e38f };
+        int best_sh[2] = { 0, 0 }, best_grid[2] = { 0, 0 };
         for (int sh = 0; sh < (c->mixed ? NFSHAPE_MIXED : NFSHAPE_ALL); ++sh) {
             const int occ = flux2d_occ(c, sh);
             for (int o = occ; o >= 1 && o >= occ - 1; --o) {
@@ -1345,36 +1382,35 @@ es_status es_autotune(es_ctx* c, const double* JU, const double* J, const double
                 float ms = 0.f;
                 cudaEventElapsedTime(&ms, e0, e1);
                 ms /= (float)reps;
-                if (ms < best) {
-                    best = ms;
-                    c->fused_ms = ms;
-                    if (ms < c->flux_ms[0] + c->flux_ms[1]) {
-                        if (sh < NFSHAPE) {
-                            c->fused_shape = sh;
-                            c->fused_grid = grid;
-                        } else {
-                            if (c->fused_shape < 0) {
-                                c->fused_shape = 0;
-                                c->fused_grid = c->sms * flux2d_occ(c, 0);
-                            }
-                            c->fused_run = sh;
-                            c->fused_run_grid = grid;
-                        }
-                    }
+                const int beyond = sh < NFSHAPE ? 0 : 1;
+                if (ms < best[beyond]) {
+                    best[beyond] = ms;
+                    best_sh[beyond] = sh;
+                    best_grid[beyond] = grid;
                 }
+            }
+        }
+        c->fused_ms = best[0] < 3.0e38f ? best[0] : 0.f;
+        if (std::min(best[0], best[1]) < c->flux_ms[0] + c->flux_ms[1]) {
+            c->fused_shape = best_sh[0];
+            c->fused_grid = best_grid[0];
+            if (best[1] < best[0]) {
+                c->fused_run = best_sh[1];
+                c->fused_run_grid = best_grid[1];
+                c->fused_run_ms = best[1];
             }
         }
     }
     // mixed 2D: the fused mesh-step launch in each tile shape, after the passes it reads
     // (metrics, CFL and monitor gradients) on the same state; it writes only scratch
-    c->jf_ms = 0.f;
+    c->jf_ms = c->jf_run_ms = 0.f;
     c->jf_run = -1;
     if (fused_mesh2d(c)) {
         StagePtrs Q = P;
         Q.xdot = nullptr;
         launch_metrics(c, Q, tab, st, true, false, false);
         launch_cfl_grad(c->mixed, c->d, c->N, node_grid(c, c->n_cell), st, c->dI, P, tab, c->w_cell, c->n_cell, c->dS);
-        float best = 3.0e38f;
+        float best = 3.0e38f, beyond = 3.0e38f;
         for (int sh = 0; sh < NJF_SHAPE_ALL; ++sh) {
             launch_fused_mesh2d(c, sh, P, tab, st);
             cudaEventRecord(e0, st);
@@ -1384,13 +1420,14 @@ es_status es_autotune(es_ctx* c, const double* JU, const double* J, const double
             float ms = 0.f;
             cudaEventElapsedTime(&ms, e0, e1);
             ms /= (float)reps;
-            if (ms < best) {
-                best = ms;
-                c->jf_ms = ms;
-                if (sh < NJF_SHAPE) c->jf_shape = sh;
-                else c->jf_run = sh;
+            float& b = sh < NJF_SHAPE ? best : beyond;
+            if (ms < b) {
+                b = ms;
+                (sh < NJF_SHAPE ? c->jf_shape : c->jf_run) = sh;
+                (sh < NJF_SHAPE ? c->jf_ms : c->jf_run_ms) = ms;
             }
         }
+        if (!(beyond < best)) c->jf_run = -1;
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -1427,9 +1464,8 @@ es_status es_get_tuning(const es_ctx* c, int* shape, int* S, int* WT, int* grid,
     for (int k = 0; k < 3; ++k) {
         const bool on = k < c->d;
         shape[k] = on ? c->flux_shape[k] : 0;
-        const int sh = on && c->flux_fit[k] ? NSHAPE : c->flux_shape[k];
-        S[k] = on ? shape_S(c, k, sh) : 0;
-        WT[k] = on ? shape_WT(c, k, sh) : 0;
+        S[k] = on ? SHAPE_S[c->flux_shape[k]] : 0;
+        WT[k] = on ? SHAPE_WT[c->flux_shape[k]] : 0;
         grid[k] = on ? c->flux_grid[k] : 0;
         ms[k] = on ? c->flux_ms[k] : 0.f;
     }
@@ -1470,6 +1506,74 @@ es_status es_set_fusion(es_ctx* c, int shape, int grid)
     c->fused_grid = shape >= 0 ? (grid > 0 ? grid : c->sms * flux2d_occ(c, shape)) : 0;
     c->fused_ms = 0.f;
     c->fused_run = -1;
+    drop_run_graph(c);
+    return ES_OK;
+}
+
+es_status es_get_tiles(const es_ctx* c, int launch, int* a, int* b, int* grid, float* ms)
+{
+    if (!c || !a || !b || !grid || !ms || launch < ES_TILES_FLUX1 || launch > ES_TILES_MESH) return ES_ERR_ARG;
+    *a = *b = *grid = 0;
+    *ms = 0.f;
+    if (launch <= ES_TILES_FLUX3) {
+        const int k = launch;
+        if (k >= c->d) return ES_OK;
+        const bool fit = c->flux_fit[k];
+        *a = shape_S(c, k, fit ? NSHAPE : c->flux_shape[k]);
+        *b = shape_WT(c, k, fit ? NSHAPE : c->flux_shape[k]);
+        *grid = fit ? c->fit_grid[k] : c->flux_grid[k];
+        *ms = fit ? c->fit_ms[k] : c->flux_ms[k];
+    } else if (launch == ES_TILES_STAGE) {
+        if (c->fused_shape < 0) return ES_OK;
+        const bool run = c->fused_run >= 0;
+        const int sh = run ? c->fused_run : c->fused_shape;
+        *a = FSHAPE_TX[sh];
+        *b = FSHAPE_TY[sh];
+        *grid = run ? c->fused_run_grid : c->fused_grid;
+        *ms = run ? c->fused_run_ms : c->fused_ms;
+    } else if (fused_mesh2d(c)) {
+        const int sh = c->jf_run >= 0 ? c->jf_run : c->jf_shape;
+        *a = JF_SHAPES[sh][0];
+        *b = JF_SHAPES[sh][1];
+        *grid = node_grid(c, c->n_jf[sh]);
+        *ms = c->jf_run >= 0 ? c->jf_run_ms : c->jf_ms;
+    }
+    return ES_OK;
+}
+
+es_status es_set_tiles(es_ctx* c, int launch, int a, int b, int grid)
+{
+    if (!c) return ES_ERR_ARG;
+    if (launch < ES_TILES_FLUX1 || launch > ES_TILES_MESH || grid < 0) return fail(c, ES_ERR_ARG, "es_set_tiles: bad launch or negative grid");
+    if (launch <= ES_TILES_FLUX3) {
+        const int k = launch;
+        for (int sh = 0; sh < NSHAPE; ++sh)
+            if (a == SHAPE_S[sh] && b == SHAPE_WT[sh]) return es_set_tuning(c, k, sh, grid);
+        if (k >= c->d || c->d != 3 || c->mixed || a < 1 || b < 1 || b > FLUX_WT_MAX || (long long)(a + 1LL) * b > FLUX_TPB)
+            return fail(c, ES_ERR_ARG, "es_set_tiles: no flux tile of this extent");
+        if (!fit_extent(c, k, a, b)) return fail(c, ES_ERR_CUDA, "es_set_tiles: allocation failed");
+        c->flux_fit[k] = true;
+        c->fit_grid[k] = grid > 0 ? grid : shape_grid(c, k, NSHAPE);
+        c->fit_ms[k] = 0.f;
+    } else if (launch == ES_TILES_STAGE) {
+        if (a == 0 && b == 0) return es_set_fusion(c, -1, 0);
+        int sh = 0;
+        while (sh < (c->mixed ? NFSHAPE_MIXED : NFSHAPE_ALL) && !(a == FSHAPE_TX[sh] && b == FSHAPE_TY[sh])) ++sh;
+        if (c->d != 2 || sh == (c->mixed ? NFSHAPE_MIXED : NFSHAPE_ALL)) return fail(c, ES_ERR_ARG, "es_set_tiles: no stage tile of this extent");
+        if (sh < NFSHAPE) return es_set_fusion(c, sh, grid);
+        if (c->fused_shape < 0) es_set_fusion(c, 0, 0);
+        c->fused_run = sh;
+        c->fused_run_grid = grid > 0 ? grid : c->sms * flux2d_occ(c, sh);
+        c->fused_run_ms = 0.f;
+    } else {
+        int sh = 0;
+        while (sh < NJF_SHAPE_ALL && !(a == JF_SHAPES[sh][0] && b == JF_SHAPES[sh][1])) ++sh;
+        if (sh == NJF_SHAPE_ALL || !c->mixed || c->d != 2)
+            return fail(c, ES_ERR_ARG, "es_set_tiles: no mesh tile of this extent or not a mixed-form 2D context");
+        if (sh < NJF_SHAPE) return es_set_mesh_tiles(c, sh);
+        c->jf_run = sh;
+        c->jf_run_ms = 0.f;
+    }
     drop_run_graph(c);
     return ES_OK;
 }

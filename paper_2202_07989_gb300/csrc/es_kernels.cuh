@@ -17,8 +17,8 @@ constexpr int SHAPE_S[NSHAPE] = { 62, 58, 122, 30, 26, 14 };
 constexpr int SHAPE_WT[NSHAPE] = { 4, 4, 2, 8, 8, 16 };
 constexpr int SHAPE_DEFAULT_K0 = 0;    // direction 1: 62 nodes along the line x 4 lines
 constexpr int SHAPE_DEFAULT_KN = 3;    // directions 2, 3: 30 nodes x 8 neighbouring lines (coalesced)
-// fused 2D stage tiles (both directions in one launch): TX x TY output nodes, at most 256
-// interfaces per direction; the autotuner picks one shape, or the per-direction launches.  The
+// fused 2D stage tiles (both directions in one launch): TX x TY output nodes, in the five shapes of
+// the table at most 256 interfaces per direction; the autotuner picks one shape, or the per-direction launches.  The
 // shapes from NFSHAPE on are for small grids: a grid of few tiles is bound by the time one tile
 // takes, not by the chip, and a smaller tile takes less.  FSHAPE_COST is the time of one wave of
 // CTAs in each shape relative to 16 x 12 tiles, binary32 and binary64, measured on grids of one wave
@@ -28,8 +28,8 @@ constexpr int SHAPE_DEFAULT_KN = 3;    // directions 2, 3: 30 nodes x 8 neighbou
 constexpr int NFSHAPE = 5;
 // The last two are for the FP64 form only, whose phases cost whole warps on each of the SM's four
 // FP64 pipes: 16 x 14 tiles need no more rounds than 16 x 12 for 17% more nodes (two of interfaces a
-// direction, at 93% instead of 80% of their lanes: 256^2 364 -> 286 us), and 24 x 15 end some grids on
-// a full wave.
+// direction, at 93% instead of 80% of their lanes: 256^2 364 -> 286 us), and 24 x 15, with 375
+// interfaces a direction in two rounds of the 256 threads, end some grids on a full wave.
 constexpr int NFSHAPE_ALL = 10, NFSHAPE_MIXED = 8;
 constexpr int FSHAPE_TX[NFSHAPE_ALL] = { 16, 12, 14, 24, 20, 8, 12, 16, 16, 24 };
 constexpr int FSHAPE_TY[NFSHAPE_ALL] = { 12, 16, 14, 8, 10, 8, 8, 8, 14, 15 };

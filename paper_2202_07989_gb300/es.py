@@ -74,6 +74,8 @@ def lib():
             "es_set_fusion": (C.c_int, [vp, C.c_int, C.c_int]),
             "es_get_mesh_tiles": (C.c_int, [vp, ip, ip, ip, ip, C.POINTER(C.c_float)]),
             "es_set_mesh_tiles": (C.c_int, [vp, C.c_int]),
+            "es_get_tiles": (C.c_int, [vp, C.c_int, ip, ip, ip, C.POINTER(C.c_float)]),
+            "es_set_tiles": (C.c_int, [vp, C.c_int, C.c_int, C.c_int, C.c_int]),
             "entropy_production": (C.c_int, [vp, dp, dp, dp, dp, dp, vp]),
             "es_bind_batch": (C.c_int, [vp, C.POINTER(vp), C.POINTER(vp), C.POINTER(vp), C.POINTER(vp), C.POINTER(vp)]),
             "es_step_batch": (C.c_int, [vp, vp]),
@@ -286,6 +288,20 @@ class Context:
     def es_set_mesh_tiles(self, shape: int):
         """Fused mixed 2D mesh-step launch in tile shape `shape` (0..3)."""
         self._chk(self.L.es_set_mesh_tiles(self.h, int(shape)), "es_set_mesh_tiles")
+
+    # the launches of es_get_tiles / es_set_tiles: flux per direction, fused 2D stage, mixed 2D mesh step
+    TILES = ("flux_k1", "flux_k2", "flux_k3", "stage", "mesh")
+
+    def es_get_tiles(self, launch: str):
+        """(extent a, extent b, CTAs, measured ms) that a launch of TILES runs on; zeros if none."""
+        a = [C.c_int() for _ in range(3)]
+        ms = C.c_float()
+        self._chk(self.L.es_get_tiles(self.h, self.TILES.index(launch), *[C.byref(v) for v in a], C.byref(ms)), "es_get_tiles")
+        return tuple(v.value for v in a) + (ms.value,)
+
+    def es_set_tiles(self, launch: str, a: int, b: int, grid: int = 0):
+        """Run a launch of TILES on tiles of extent a x b (as es_get_tiles reports them)."""
+        self._chk(self.L.es_set_tiles(self.h, self.TILES.index(launch), int(a), int(b), int(grid)), "es_set_tiles")
 
     def es_schlieren(self, JU, J, x, psi1: float = 30.0, psi2: float = 150.0, phi=None):
         """Schlieren function of Eq. (schlieren) at the nodes."""

@@ -98,3 +98,127 @@ def test_library_grid_is_reported(form):
                 ns, lines = -(-n[k] // S), -(-n[1 if k == 0 else 0] // WT) * n[1 if k == 2 else 2]
                 spread = n[k] % S != 0 and ns * lines > grid
                 assert not spread or math.gcd(grid, ns) == 1, (n, shape, k, S, WT, grid)
+
+
+# every tile the library has: stage tiles (both forms, FP64 only) and mesh tiles
+STAGE_TILES = ((16, 12), (12, 16), (14, 14), (24, 8), (20, 10), (8, 8), (12, 8), (16, 8))
+STAGE_TILES_FP64 = ((16, 14), (24, 15))
+MESH_TILES = ((32, 8), (32, 16), (24, 16), (24, 12), (16, 8), (8, 8))
+
+
+def _same(a, b):
+    return all(bool((u == v).all()) for u, v in zip(a, b))
+
+
+@pytest.mark.parametrize("form", [0, 1])
+@pytest.mark.parametrize("d,N,n", [(2, 1, (64, 64, 1)), (2, 2, (150, 75, 1)), (3, 1, (63, 17, 10))])
+def test_tuning_round_trip(d, N, n, form):
+    """The tiles that an autotuned context runs, read with es_get_tiles and set on a new context,
+    are the tiles that one runs, with the same results; and the table's calls stay consistent: the
+    shape, extent and grid of es_get_tuning, es_get_fusion and es_get_mesh_tiles, set on another
+    context, are reported there again."""
+    torch = need_gpu()
+    pb, JU, J, x, xdot = case(d, N, n[:d], "mixed", es=True, seed=81 + N, jump=True)
+    pb = pb.with_(mu=5, nf=3, sigma=(W.SIG_RHO1, W.SIG_P), alpha=(60.0, 25.0))
+    G = [to_dev(t, torch) for t in (JU, J, x)]
+    a, b, t = _ctx(pb, form), _ctx(pb, form), _ctx(pb, form)
+    untuned = a.es_step(*[g.clone() for g in G])
+    a.es_autotune(*G, None, reps=2)
+    for launch in b.TILES:
+        TX, TY, grid, ms = a.es_get_tiles(launch)
+        runs = (launch != "flux_k3" or d == 3) and (launch != "stage" or d == 2) and (launch != "mesh" or (d == 2 and form == 1))
+        assert (TX > 0 and ms > 0) == (runs and (launch != "stage" or a.es_get_fusion()[0] >= 0)), launch
+        if TX or (launch == "stage" and d == 2):
+            b.es_set_tiles(launch, TX, TY, grid)
+        assert b.es_get_tiles(launch)[:3] == (TX, TY, grid), launch
+    assert _same(a.es_step(*[g.clone() for g in G]), untuned) and _same(b.es_step(*[g.clone() for g in G]), untuned)
+    for k, (sh, S, WT, grid, ms) in enumerate(a.es_get_tuning()):
+        t.es_set_tuning(k, sh, grid)
+        assert t.es_get_tuning()[k][:4] == (sh, S, WT, grid) and t.es_get_tiles("flux_k%d" % (k + 1))[:3] == (S, WT, grid) and ms > 0
+        if a.es_get_tiles("flux_k%d" % (k + 1))[:2] != (S, WT):
+            assert a.es_get_tiles("flux_k%d" % (k + 1))[3] < ms
+    if d == 2:
+        sh, TX, TY, grid, ms = a.es_get_fusion()
+        t.es_set_fusion(sh, grid)
+        assert t.es_get_fusion()[:4] == (sh, TX, TY, grid) == (sh,) + t.es_get_tiles("stage")[:3] and ms > 0
+        if a.es_get_tiles("stage")[:2] != (TX, TY):
+            assert a.es_get_tiles("stage")[3] < ms
+    if d == 2 and form == 1:
+        sh, TX, TY, thr, ms = a.es_get_mesh_tiles()
+        t.es_set_mesh_tiles(sh)
+        assert t.es_get_mesh_tiles()[:4] == (sh, TX, TY, thr) and t.es_get_tiles("mesh")[:2] == (TX, TY) and ms > 0
+
+
+@pytest.mark.parametrize("form", [0, 1])
+@pytest.mark.parametrize("N", [1, 2])
+@pytest.mark.parametrize("weno,es_", [(0, True), (1, True), (0, False)])
+def test_every_stage_tile_bitwise(form, N, weno, es_):
+    """Every stage tile, 24 x 15 with its 375 interfaces a direction among them, gives the residual
+    of the per-direction launches bit for bit on ragged, sub-tile and several-wave grids."""
+    torch = need_gpu()
+    for n, bc, seed in (((70, 37), "mixed", 91), ((10, 11), "reflect", 92), ((349, 151), "mixed", 93), ((33, 300), "periodic", 94)):
+        pb, JU, J, x, xdot = case(2, N, n, bc, es=es_, seed=seed + N, jump=True)
+        ctx = _ctx(pb.with_(weno=weno), form)
+        G = [to_dev(t, torch) for t in (JU, J, x, xdot)]
+        ctx.es_set_tiles("stage", 0, 0)
+        assert ctx.es_get_fusion()[0] == -1
+        ref = ctx.es_rhs(*G)
+        for tile in STAGE_TILES + (STAGE_TILES_FP64 if form == 0 else ()):
+            for grid in (0, 152):
+                ctx.es_set_tiles("stage", *tile, grid)
+                assert ctx.es_get_tiles("stage")[:2] == tile and grid in (0, ctx.es_get_tiles("stage")[2])
+                assert _same(ctx.es_rhs(*G), ref), (n, tile, grid)
+
+
+@pytest.mark.parametrize("bc", ["periodic", "mixed", "reflect"])
+@pytest.mark.parametrize("mu,nf", [(1, 0), (5, 3), (8, 4), (9, 3), (16, 4), (3, 6)])
+def test_every_mesh_tile_bitwise(bc, mu, nf):
+    """Every mesh tile gives the mesh velocity and Delta t / Delta tau of the 32 x 8 tiles bit for bit."""
+    torch = need_gpu()
+    for n, seed in (((70, 37), 95), ((10, 11), 96), ((200, 199), 97)):
+        pb, JU, J, x, _ = case(2, 2, n, bc, es=True, seed=seed, jump=True)
+        ctx = _ctx(pb.with_(mu=mu, nf=nf, sigma=(W.SIG_RHO1, W.SIG_P), alpha=(60.0, 25.0)), 1)
+        G = [to_dev(t, torch) for t in (JU, J, x)]
+        ref = None
+        for tile in MESH_TILES:
+            ctx.es_set_tiles("mesh", *tile)
+            assert ctx.es_get_tiles("mesh")[:2] == tile
+            out = ctx.mesh_redistribute(*G)
+            ref = ref or out
+            assert _same(out, ref), (n, tile)
+
+
+@pytest.mark.parametrize("N", [1, 2])
+def test_fp64_3d_extents_bitwise(N):
+    """FP64 3D flux tiles of any extent, the longest segment (255 x 1) and the most lines (15 x 16)
+    among them, give the residual of the table's shape bit for bit."""
+    torch = need_gpu()
+    for n, seed in (((260, 10, 11), 98), ((10, 33, 130), 99)):
+        pb, JU, J, x, xdot = case(3, N, n, "mixed", es=True, seed=seed, jump=True)
+        ctx = _ctx(pb, 0)
+        G = [to_dev(t, torch) for t in (JU, J, x, xdot)]
+        for k in range(3):
+            ctx.es_set_tuning(k, 0)
+        ref = ctx.es_rhs(*G)
+        for tile in ((255, 1), (15, 16), (1, 16), (1, 1), (127, 2), (50, 5), (7, 13), (255, 1)):
+            for k in range(3):
+                ctx.es_set_tiles("flux_k%d" % (k + 1), *tile)
+                assert ctx.es_get_tiles("flux_k%d" % (k + 1))[:2] == tile
+            assert _same(ctx.es_rhs(*G), ref), (n, tile)
+
+
+def test_tiles_refused():
+    """Extents without a tile, launches that do not exist and forms without the launch are refused."""
+    need_gpu()
+    from paper_2202_07989_gb300 import es
+    c2, f2 = _ctx(W.random_problem(2, 1, (20, 20)), 1), _ctx(W.random_problem(2, 1, (20, 20)), 0)
+    c3, f3 = _ctx(W.random_problem(3, 1, (20, 20, 20)), 1), _ctx(W.random_problem(3, 1, (20, 20, 20)), 0)
+    for ctx, launch, a, b in ((c2, "stage", 16, 14), (c2, "stage", 9, 9), (c2, "stage", 8, 0), (c3, "stage", 16, 12), (c2, "flux_k3", 62, 4),
+                              (c2, "flux_k1", 61, 4), (f2, "flux_k1", 61, 4), (c3, "flux_k1", 61, 4), (f3, "flux_k1", 256, 1),
+                              (f3, "flux_k2", 0, 4), (f3, "flux_k2", 4, 0), (f3, "flux_k2", 14, 17), (f3, "flux_k3", 16, 16),
+                              (f3, "flux_k1", 2 ** 31 - 1, 2), (f2, "mesh", 32, 8), (c3, "mesh", 32, 8), (c2, "mesh", 9, 9)):
+        with pytest.raises(es.EsError):
+            ctx.es_set_tiles(launch, a, b)
+    with pytest.raises(es.EsError):
+        c2.es_set_tiles("stage", 8, 8, -1)
+    assert c2.L.es_set_tiles(c2.h, 5, 8, 8, 0) == 1 and c2.L.es_set_tiles(None, 3, 8, 8, 0) == 1
