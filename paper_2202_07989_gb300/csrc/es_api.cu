@@ -730,15 +730,14 @@ bool fused_mesh2d(const es_ctx* c)
     return c->mixed && c->d == 2 && !I.fixed && I.mu >= 1;
 }
 
-// The mesh tiles of a context that nobody tuned: least time by the model of JF_COST.  The
+// The mesh tiles of a context that nobody tuned: least time by the model of jf_cost.  The
 // arithmetic is the same in every shape.
 void pick_mesh_tiles(es_ctx* c)
 {
+    if (!fused_mesh2d(c)) return;
     double best = 0.0;
     for (int sh = 0; sh < NJF_SHAPE_ALL; ++sh) {
-        if (JF_COST[sh] <= 0.0) continue;
-        const int per_sm = (c->n_jf[sh] + c->sms - 1) / c->sms;
-        const double t = JF_COST[sh] * (1.3 * (per_sm / 2) + per_sm % 2);
+        const double t = jf_cost(sh, c->hI[0].mu, c->hI[0].nf, c->n_jf[sh], c->sms);
         if (c->jf_run < 0 || t < best) {
             best = t;
             c->jf_run = sh;

@@ -1101,6 +1101,32 @@ size_t jacobi_fused2d_smem(int H, int F, int shape)
     return sizeof(float) * (17 * nr + 2 * nro);
 }
 
+// A launch takes a tile's chain of phases (per thread: slots of the outer region for the filter passes,
+// of the inner one for the spacings and each sweep) once per wave of resident tiles, and each tile adds
+// what it issues.  Resident: 1024 threads per SM at the kernel's registers, and the shared memory, which
+// holds one 32 x 16 tile of 8 sweeps and 4 passes.  Coefficients: least squares over 897 mesh steps of 23
+// grids (32^2 .. 1000^2, 2000 x 400) with mu = 1..8, 10, 16 and nf = 0..6 in every shape; the shape of
+// least modelled time was within 0.4% of the fastest on average, 9% at most.  A rule by the tile
+// count alone took 32 x 16 tiles for 8 sweeps a launch: mesh step of 1200 x 480 with mu = 8, nf = 4
+// 271 us where 24 x 16 take 235, with mu = 16 413 where they take 352.
+double jf_cost(int sh, int mu, int nf, int tiles, int sms)
+{
+    const int TX = JF_SHAPES[sh][0], TY = JF_SHAPES[sh][1], TPB = JF_SHAPES[sh][2], np = jf_passes(mu);
+    double t = 0.0;
+    for (int p = 0, done = 0; p < np; ++p) {
+        const int H = jf_sweeps(mu, np, p, done), F = p == 0 && nf <= FILTER_FUSED_MAX ? nf : 0;
+        done += H;
+        const double NR = (TX + 2 * H) * (TY + 2 * H), NRo = (TX + 2 * H + 2 * F) * (TY + 2 * H + 2 * F);
+        const int by_smem = (int)(228 * 1024 / (jacobi_fused2d_smem(H, F, sh) + 1280)), R = by_smem < 1024 / TPB ? by_smem : 1024 / TPB;
+        const double wave = 3.41 + 0.134 * F * NRo / TPB + (1.454 + 0.067 * H) * NR / TPB;
+        const double issue = 1e-3 * (0.698 * TPB + 0.18 * F * NRo + 0.318 * H * NR + 4.689 * TX * TY);
+        const int m = (tiles + sms - 1) / sms;      // tiles of the fullest SM
+        const double per = (double)tiles / sms;
+        t += m > 4 * R ? per * (wave / R + issue) : (m + R - 1) / R * wave + m * issue;
+    }
+    return t + (sh == JF_SHAPE_DEFAULT ? 0.0 : 1.5);     // another shape only for more than 1.5 us
+}
+
 #define JF_KERNELS(X) X(0, 32, 8, 256) X(1, 32, 16, 512) X(2, 24, 16, 512) X(3, 24, 12, 512) X(4, 16, 8, 512) X(5, 8, 8, 512)
 
 void prepare_mesh()
@@ -1129,11 +1155,10 @@ static void launch_jacobi_fused2d(int shape, int grid, cudaStream_t st, const In
 void jacobi_fused2d(int shape, int grid, cudaStream_t st, const Inst* insts, const StagePtrs& single,
                     const StagePtrs* table, const int2* work, int nwork, const Scratch* scr, int mu, int F, int theta_sel)
 {
-    // launches of at most JACOBI_FUSED_MAX sweeps, as equal as they come; y alternates between the
-    // two buffers and ends in the one xmu_of names
-    const int np = (mu + JACOBI_FUSED_MAX - 1) / JACOBI_FUSED_MAX;
+    // y alternates between the two buffers and ends in the one xmu_of names
+    const int np = jf_passes(mu);
     for (int p = 0, done = 0; p < np; ++p) {
-        const int H = (mu - done + np - p - 1) / (np - p), left = np - 1 - p;
+        const int H = jf_sweeps(mu, np, p, done), left = np - 1 - p;
         const int end = mu % 2 == 1 ? 1 : 2, dst = left % 2 == 0 ? end : 3 - end;
         JfPass pass;
         pass.src = p == 0 ? 0 : 3 - dst;

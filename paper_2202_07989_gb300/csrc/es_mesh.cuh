@@ -115,19 +115,20 @@ constexpr int JACOBI_FUSED_MAX = 8, FILTER_FUSED_MAX = 4;
 constexpr int NJF_SHAPE = 4;
 // The shapes from NJF_SHAPE on are for small grids, where the time one tile takes counts (its
 // slots per thread: 16 x 8 tiles with 512 threads have one per sweep at mu = 5, 32 x 8 with 256
-// three).  JF_COST: microseconds of a launch of mu = 5, n_f = 3 with at most one tile per SM; two
-// resident tiles take 1.3 times as long (measured; shapes 0-3 of one wave 19, 19, 17, 16.5 us).
-// A context that nobody tuned takes the shape of least time by that model (pick_mesh_tiles in
-// es_api.cu): measured mesh steps, 32 x 8 tiles against the model's choice: 64^2 (mu = 10) 57.2 ->
-// 39.7 us, 200 x 100 38.4 -> 32.8, 350 x 150 43.3 -> 39.6, 800 x 160 64.8 -> 55.3, 1200 x 480 203 -> 169
+// three).  A context that nobody tuned takes the shape of least time by the model of jf_cost.
 constexpr int NJF_SHAPE_ALL = 6;
 constexpr int JF_SHAPES[NJF_SHAPE_ALL][3] = { { 32, 8, 256 }, { 32, 16, 512 }, { 24, 16, 512 }, { 24, 12, 512 },
                                               { 16, 8, 512 }, { 8, 8, 512 } };
-constexpr double JF_COST[NJF_SHAPE_ALL] = { 0.0, 19.0, 17.0, 16.5, 11.4, 10.3 };    // 0: never the model's choice
 constexpr int JF_SHAPE_DEFAULT = 0;
 void prepare_mesh();    // kernel attributes, once per context
 void prepare_mesh3d();  // those of es_mesh3d.cu
 size_t jacobi_fused2d_smem(int H, int F, int shape);
+// microseconds (up to a constant of the grid) of the fused launches of a mesh step with mu sweeps and
+// nf filter passes over `tiles` tiles of shape sh on `sms` SMs
+double jf_cost(int sh, int mu, int nf, int tiles, int sms);
+// sweeps of launch p of np after `done` of mu: at most JACOBI_FUSED_MAX, as equal as they come
+inline int jf_passes(int mu) { return (mu + JACOBI_FUSED_MAX - 1) / JACOBI_FUSED_MAX; }
+inline int jf_sweeps(int mu, int np, int p, int done) { return (mu - done + np - p - 1) / (np - p); }
 // one launch of several: the displacement buffer it starts from (0: y = 0, 1: xa, 2: xb) and ends
 // in, whether it stores Theta for the next one, and whether it is the last (limiter bounds).
 // edges: at the grid's first and last nodes the passes keep the order of operations in which a step

@@ -222,3 +222,46 @@ def test_tiles_refused():
     with pytest.raises(es.EsError):
         c2.es_set_tiles("stage", 8, 8, -1)
     assert c2.L.es_set_tiles(c2.h, 5, 8, 8, 0) == 1 and c2.L.es_set_tiles(None, 3, 8, 8, 0) == 1
+
+
+@pytest.mark.parametrize("n,mu,nf", [((64, 64), 1, 0), ((64, 64), 8, 4), ((200, 100), 3, 0), ((400, 200), 8, 0), ((400, 200), 8, 4),
+                                     ((1200, 480), 1, 4), ((1200, 480), 3, 3), ((1200, 480), 8, 0), ((1200, 480), 8, 4),
+                                     ((1200, 480), 16, 4)])
+def test_untuned_mesh_tiles_speed(n, mu, nf):
+    """The mesh tiles that an untuned context picks for its grid, sweeps and filter passes take no
+    more than 8% longer than the best tiles (a mesh step's time comes in steps of about 2 us, up to
+    7% of the smallest ones here)."""
+    torch = need_gpu()
+    pb, U, x = W.shock_bubble_2d(*n)
+    ctx = _ctx(pb.with_(mu=mu, nf=nf), 1)
+    xg = to_dev(x, torch)
+    J = ctx.es_init_mesh(xg)
+    JU = to_dev(U, torch) * J
+    xd, dd = torch.empty_like(xg), torch.empty(2, dtype=torch.float64, device="cuda")
+
+    def us():
+        st = torch.cuda.Stream()
+        with torch.cuda.stream(st):
+            ctx.mesh_redistribute(JU, J, xg, xdot=xd, dt_dtau=dd)
+            st.synchronize()
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=st):
+                ctx.mesh_redistribute(JU, J, xg, xdot=xd, dt_dtau=dd)
+            best = float("inf")
+            for _ in range(6):
+                e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+                g.replay()
+                e[0].record(st)
+                for _ in range(10):
+                    g.replay()
+                e[1].record(st)
+                e[1].synchronize()
+                best = min(best, 100 * e[0].elapsed_time(e[1]))
+        return best
+
+    picked, t = ctx.es_get_tiles("mesh")[:2], us()
+    all_ = {}
+    for tile in MESH_TILES:
+        ctx.es_set_tiles("mesh", *tile)
+        all_[tile] = us()
+    assert t <= 1.08 * min(all_.values()), (picked, t, all_)
