@@ -243,7 +243,8 @@ es_status es_set_mesh_tiles(es_ctx* ctx, int shape);
  * has: the shapes above and those beyond them.  launch: the flux launch of direction
  * 1..3 (a = S nodes along the line, b = WT lines; 2D contexts run it only without the
  * fused stage launch), the fused 2D stage launch (a = TX, b = TY) or the mixed 2D mesh
- * step (a = TX, b = TY).  No tile changes a result.
+ * step (a = TX, b = TY; 1 x 1: one launch per filter pass and sweep, for more than
+ * 8 sweeps or 4 filter passes).  No tile changes a result.
  * es_get_tiles: the extent, the CTAs and the time the last es_autotune measured for
  * them (0 if none; mesh step: all its monitor, filter and sweep launches); zeros for a
  * launch the context does not run.  All pointers HOST, one value each.

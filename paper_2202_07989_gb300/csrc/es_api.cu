@@ -730,8 +730,11 @@ bool fused_mesh2d(const es_ctx* c)
     return c->mixed && c->d == 2 && !I.fixed && I.mu >= 1;
 }
 
-// The mesh tiles of a context that nobody tuned: least time by the model of jf_cost.  The
-// arithmetic is the same in every shape.
+// whether the mixed 2D mesh step may run one launch per filter pass and sweep
+bool may_per_sweep(const es_ctx* c) { return fused_mesh2d(c) && (c->hI[0].mu > JACOBI_FUSED_MAX || c->hI[0].nf > FILTER_FUSED_MAX); }
+
+// The mesh tiles of a context that nobody tuned: least time by the models of jf_cost and
+// per_sweep_cost.  The arithmetic is the same in all of them.
 void pick_mesh_tiles(es_ctx* c)
 {
     if (!fused_mesh2d(c)) return;
@@ -743,18 +746,24 @@ void pick_mesh_tiles(es_ctx* c)
             c->jf_run = sh;
         }
     }
+    if (may_per_sweep(c) && per_sweep_cost(c->hI[0].mu, c->hI[0].nf, c->n_cell) < best) c->jf_run = JF_PER_SWEEP;
 }
 
-// the fused 2D launches of a mesh step in tile shape js; more filter passes than they hold run
-// as launches of their own before them
+// the launches of a mixed 2D mesh step in tile shape js (or JF_PER_SWEEP); more filter passes than
+// the fused ones hold run as launches of their own before them
 void launch_fused_mesh2d(es_ctx* c, int js, const StagePtrs& P, const StagePtrs* tab, cudaStream_t st)
 {
     const int mu = c->hI[0].mu, nf = c->hI[0].nf, gc = node_grid(c, c->n_cell);
     int F = nf;
-    if (nf > FILTER_FUSED_MAX) {
+    if (nf > FILTER_FUSED_MAX || js == JF_PER_SWEEP) {
         launch_monitor_theta(true, gc, st, c->dI, c->w_cell, c->n_cell, c->dS);
         for (int f = 0; f < nf; ++f) launch_filter(true, false, gc, st, c->dI, c->w_cell, c->n_cell, c->dS, f % 2);
         F = -1;
+    }
+    if (js == JF_PER_SWEEP) {
+        for (int s = 0; s < mu; ++s)
+            launch_jacobi_y2d(s == 0, s == mu - 1, gc, st, c->dI, P, tab, c->w_cell, c->n_cell, c->dS, s, nf % 2);
+        return;
     }
     jacobi_fused2d(js, node_grid(c, c->n_jf[js]), st, c->dI, P, tab, c->w_jf[js], c->n_jf[js], c->dS, mu, F, nf % 2);
 }
@@ -1410,7 +1419,7 @@ es_status es_autotune(es_ctx* c, const double* JU, const double* J, const double
         launch_metrics(c, Q, tab, st, true, false, false);
         launch_cfl_grad(c->mixed, c->d, c->N, node_grid(c, c->n_cell), st, c->dI, P, tab, c->w_cell, c->n_cell, c->dS);
         float best = 3.0e38f, beyond = 3.0e38f;
-        for (int sh = 0; sh < NJF_SHAPE_ALL; ++sh) {
+        for (int sh = 0; sh < NJF_SHAPE_ALL + may_per_sweep(c); ++sh) {
             launch_fused_mesh2d(c, sh, P, tab, st);
             cudaEventRecord(e0, st);
             for (int r = 0; r < reps; ++r) launch_fused_mesh2d(c, sh, P, tab, st);
@@ -1534,7 +1543,7 @@ es_status es_get_tiles(const es_ctx* c, int launch, int* a, int* b, int* grid, f
         const int sh = c->jf_run >= 0 ? c->jf_run : c->jf_shape;
         *a = JF_SHAPES[sh][0];
         *b = JF_SHAPES[sh][1];
-        *grid = node_grid(c, c->n_jf[sh]);
+        *grid = node_grid(c, sh == JF_PER_SWEEP ? c->n_cell : c->n_jf[sh]);
         *ms = c->jf_run >= 0 ? c->jf_run_ms : c->jf_ms;
     }
     return ES_OK;
@@ -1566,8 +1575,9 @@ es_status es_set_tiles(es_ctx* c, int launch, int a, int b, int grid)
         c->fused_run_ms = 0.f;
     } else {
         int sh = 0;
-        while (sh < NJF_SHAPE_ALL && !(a == JF_SHAPES[sh][0] && b == JF_SHAPES[sh][1])) ++sh;
-        if (sh == NJF_SHAPE_ALL || !c->mixed || c->d != 2)
+        const int n = NJF_SHAPE_ALL + may_per_sweep(c);
+        while (sh < n && !(a == JF_SHAPES[sh][0] && b == JF_SHAPES[sh][1])) ++sh;
+        if (sh == n || !c->mixed || c->d != 2)
             return fail(c, ES_ERR_ARG, "es_set_tiles: no mesh tile of this extent or not a mixed-form 2D context");
         if (sh < NJF_SHAPE) return es_set_mesh_tiles(c, sh);
         c->jf_run = sh;

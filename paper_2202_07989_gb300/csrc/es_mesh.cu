@@ -792,6 +792,136 @@ __global__ void jacobi_kernel(const Inst* __restrict__ insts, StagePtrs single, 
     }
 }
 
+// Mixed form, 2D: one Jacobi sweep of the mesh equation on the displacement y = x - x^n in
+// binary32, for the mesh steps that run one launch per filter pass and sweep (JF_PER_SWEEP).
+// With the spacings dl_{k+-} = x^n_{i+-e_k} - x^n_i (formed in FP64 by the first sweep, stored
+// rounded to binary32) the sweep x_i <- sum T_{k+-} x_{i+-e_k} / dxi_k^2 / sum T_{k+-} / dxi_k^2
+// reads y_i <- sum w_{k+-} (dl_{k+-} + y_{i+-e_k}) / sum w_{k+-}.
+// The positions stay FP64 (x^n + y); only the sweep arithmetic is FP32.  The last sweep
+// also forms the limiter bounds of Sec. 4, dl_{k,s}[k] / (2 y_k) with s the sign of y_k.
+template <bool FIRST, bool LAST>
+__global__ void __launch_bounds__(NODE_TPB) jacobi_y_kernel(const Inst* __restrict__ insts, StagePtrs single,
+                                                             const StagePtrs* __restrict__ table,
+                                                             const int2* __restrict__ work, int nwork,
+                                                             const Scratch* __restrict__ scr, int sweep, int theta_sel)
+{
+    constexpr int D = 2;
+    pdl_entry();
+    __shared__ double sh[32];
+    for (int wi = blockIdx.x; wi < nwork; wi += gridDim.x) {
+        const int2 it = work[wi];
+        const Inst& I = insts[it.x];
+        int i[3];
+        const bool valid = tile_node(I, it.y, 0, i[0], i[1], i[2]);
+        ES_PTRS(P);
+        float bnd = 1.0f;
+        if (valid) {
+            const Scratch& Sc = scr[it.x];
+            const long long n = I.ncell;
+            const long long p = lin(I, i[0], i[1], i[2]);
+            const float* th = reinterpret_cast<const float*>(theta_sel ? Sc.th1 : Sc.th0);
+            const float* ys = reinterpret_cast<const float*>(sweep % 2 == 1 ? Sc.xa : Sc.xb);
+            float* yd = reinterpret_cast<float*>(sweep % 2 == 0 ? Sc.xa : Sc.xb);
+            float* dl = Sc.dl;
+            const float tc = th[p];
+            bool inner = true;
+#pragma unroll
+            for (int k = 0; k < D; ++k) inner = inner && i[k] >= 1 && i[k] < I.n[k] - 1;
+            float num[D], den = 0.0f, dk[D][2];
+#pragma unroll
+            for (int j = 0; j < D; ++j) num[j] = 0.0f;
+            if (inner && !FIRST) {
+                // interior, after the first sweep: every load up front, no boundary maps
+                const long long st[3] = { 1, I.n[0], (long long)I.n[0] * I.n[1] };
+                float tn[D][2], dv[D][2][D], yv[D][2][D];
+#pragma unroll
+                for (int k = 0; k < D; ++k)
+#pragma unroll
+                    for (int s = 0; s < 2; ++s) {
+                        const long long q = p + (s ? st[k] : -st[k]);
+                        tn[k][s] = th[q];
+#pragma unroll
+                        for (int j = 0; j < D; ++j) {
+                            dv[k][s][j] = dl[((k * 2 + s) * D + j) * n + p];
+                            yv[k][s][j] = ys[j * n + q];
+                        }
+                    }
+#pragma unroll
+                for (int k = 0; k < D; ++k)
+#pragma unroll
+                    for (int s = 0; s < 2; ++s) {
+                        const float w = 0.5f * (tc + tn[k][s]) * I.f_h2[k];
+                        dk[k][s] = dv[k][s][k];
+#pragma unroll
+                        for (int j = 0; j < D; ++j) num[j] = fmaf(w, dv[k][s][j] + yv[k][s][j], num[j]);
+                        den += w;
+                    }
+            } else {
+            long long stride = 1;
+#pragma unroll
+            for (int k = 0; k < D; ++k) {
+#pragma unroll
+                for (int s = 0; s < 2; ++s) {
+                    int nb[3] = { i[0], i[1], i[2] };
+                    nb[k] += s ? 1 : -1;
+                    const long long q = p + (s ? stride : -stride);
+                    const float w = 0.5f * (tc + th[inner ? q : s_map(I, nb[0], nb[1], nb[2])]) * I.f_h2[k];
+                    float dv[D], yv[D];
+                    if (FIRST) {
+                        double xn[3];
+                        if (inner) {
+#pragma unroll
+                            for (int j = 0; j < D; ++j) xn[j] = P.x[j * n + q];
+                        } else {
+                            x_at<false>(I, P.x, nb[0], nb[1], nb[2], xn);
+                        }
+#pragma unroll
+                        for (int j = 0; j < D; ++j) {
+                            dv[j] = f64_to_f32(xn[j] - P.x[j * n + p]);
+                            dl[((k * 2 + s) * D + j) * n + p] = dv[j];
+                            yv[j] = 0.0f;
+                        }
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < D; ++j) dv[j] = dl[((k * 2 + s) * D + j) * n + p];
+                        if (inner) {
+#pragma unroll
+                            for (int j = 0; j < D; ++j) yv[j] = ys[j * n + q];
+                        } else {
+                            y_at(I, ys, nb[0], nb[1], nb[2], yv);
+                        }
+                    }
+                    dk[k][s] = dv[k];
+#pragma unroll
+                    for (int j = 0; j < D; ++j) num[j] = fmaf(w, dv[j] + yv[j], num[j]);
+                    den += w;
+                }
+                stride *= I.n[k];
+            }
+            }
+            float ynew[D];
+#pragma unroll
+            for (int j = 0; j < D; ++j) {
+                ynew[j] = num[j] / den;
+                yd[j * n + p] = ynew[j];
+            }
+            if (LAST) {
+#pragma unroll
+                for (int k = 0; k < D; ++k) {
+                    const float dx = ynew[k];
+                    if (dx < 0.0f) bnd = fminf(bnd, dk[k][0] / (2.0f * dx));
+                    else if (dx > 0.0f) bnd = fminf(bnd, dk[k][1] / (2.0f * dx));
+                }
+                if (!(bnd >= 0.0f)) bnd = 0.0f;
+            }
+        }
+        if (LAST) {
+            const double m = block_min_pos(f32_to_f64(bnd), sh);
+            if (threadIdx.x == 0) atomic_min_pos(&scr[it.x].red[5], m);
+        }
+    }
+}
+
 // Slot q = threadIdx.x, threadIdx.x + TPB, ... of a W-wide region (TPB threads per block) and its column and row
 // (a, b) = (q % W, q / W), stepped without a division per slot (W is a run-time width)
 template <int TPB>
@@ -1125,6 +1255,18 @@ double jf_cost(int sh, int mu, int nf, int tiles, int sms)
         t += m > 4 * R ? per * (wave / R + issue) : (m + R - 1) / R * wave + m * issue;
     }
     return t + (sh == JF_SHAPE_DEFAULT ? 0.0 : 1.5);     // another shape only for more than 1.5 us
+}
+
+// Each launch takes about 3 us and what its nodes take.  Against the fused launches, measured over 22
+// grids (32^2 .. 1400^2, 2400 x 480), mu = 9..32 and nf = 0..6 (fused : per sweep, us a mesh step): mu = 10
+// 64^2 43 : 84, 400 x 200 67 : 85, 512^2 136 : 147, 1000^2 429 : 428, 2400 x 480 461 : 412; mu = 16
+// 512^2 193 : 191, 1200 x 480 353 : 331, 2000 x 400 480 : 380, 1400^2 1171 : 892.  The choice of least
+// modelled time was within 0.5% of the fastest on average, 8% at most.
+double per_sweep_cost(int mu, int nf, int tiles)
+{
+    const double n = 1e-5 * NODE_TPB * tiles;
+    const int passes = nf <= FILTER_FUSED_MAX ? nf + 1 : 0;     // (beyond that the fused ones launch Theta and passes too)
+    return 2.938 + 5.048 * n + mu * (2.472 + 0.734 * n) + passes * (3.465 + 0.873 * n) + 2.0;
 }
 
 #define JF_KERNELS(X) X(0, 32, 8, 256) X(1, 32, 16, 512) X(2, 24, 16, 512) X(3, 24, 12, 512) X(4, 16, 8, 512) X(5, 8, 8, 512)
@@ -1652,6 +1794,15 @@ void launch_xdot(bool mixed, int grid, cudaStream_t st, const Inst* insts, const
 {
     if (mixed) pdl_launch(xdot_kernel<true>, grid, NODE_TPB, 0, st, insts, single, table, work, nwork, scr);
     else pdl_launch(xdot_kernel<false>, grid, NODE_TPB, 0, st, insts, single, table, work, nwork, scr);
+}
+
+void launch_jacobi_y2d(bool first, bool last, int grid, cudaStream_t st, const Inst* insts, const StagePtrs& single,
+                       const StagePtrs* table, const int2* work, int nwork, const Scratch* scr, int sweep, int theta_sel)
+{
+#define JY(F, LS) pdl_launch(jacobi_y_kernel<F, LS>, grid, NODE_TPB, 0, st, insts, single, table, work, nwork, scr, sweep, theta_sel)
+    if (first) { if (last) JY(true, true); else JY(true, false); }
+    else { if (last) JY(false, true); else JY(false, false); }
+#undef JY
 }
 
 void launch_jacobi(bool last, int grid, cudaStream_t st, const Inst* insts, const StagePtrs& single,

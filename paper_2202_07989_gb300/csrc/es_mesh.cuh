@@ -117,8 +117,12 @@ constexpr int NJF_SHAPE = 4;
 // slots per thread: 16 x 8 tiles with 512 threads have one per sweep at mu = 5, 32 x 8 with 256
 // three).  A context that nobody tuned takes the shape of least time by the model of jf_cost.
 constexpr int NJF_SHAPE_ALL = 6;
-constexpr int JF_SHAPES[NJF_SHAPE_ALL][3] = { { 32, 8, 256 }, { 32, 16, 512 }, { 24, 16, 512 }, { 24, 12, 512 },
-                                              { 16, 8, 512 }, { 8, 8, 512 } };
+// JF_PER_SWEEP: no tiles, one launch per filter pass and sweep over the grid's nodes.  It rounds as the
+// fused launches do beyond 8 sweeps or 4 filter passes, and is a choice there: a launch costs about 4 us
+// on small grids but recomputes no halo on large ones
+constexpr int JF_PER_SWEEP = NJF_SHAPE_ALL;
+constexpr int JF_SHAPES[NJF_SHAPE_ALL + 1][3] = { { 32, 8, 256 }, { 32, 16, 512 }, { 24, 16, 512 }, { 24, 12, 512 },
+                                              { 16, 8, 512 }, { 8, 8, 512 }, { 1, 1, 256 } };
 constexpr int JF_SHAPE_DEFAULT = 0;
 void prepare_mesh();    // kernel attributes, once per context
 void prepare_mesh3d();  // those of es_mesh3d.cu
@@ -126,6 +130,8 @@ size_t jacobi_fused2d_smem(int H, int F, int shape);
 // microseconds (up to a constant of the grid) of the fused launches of a mesh step with mu sweeps and
 // nf filter passes over `tiles` tiles of shape sh on `sms` SMs
 double jf_cost(int sh, int mu, int nf, int tiles, int sms);
+// the same for one launch per filter pass and sweep over `tiles` tiles of NODE_TPB nodes
+double per_sweep_cost(int mu, int nf, int tiles);
 // sweeps of launch p of np after `done` of mu: at most JACOBI_FUSED_MAX, as equal as they come
 inline int jf_passes(int mu) { return (mu + JACOBI_FUSED_MAX - 1) / JACOBI_FUSED_MAX; }
 inline int jf_sweeps(int mu, int np, int p, int done) { return (mu - done + np - p - 1) / (np - p); }
@@ -146,6 +152,9 @@ void launch_filter3d(int grid, cudaStream_t st, const Inst* insts, const int2* w
 // mixed form, 3D: one Jacobi sweep marching along i3 over the column items of col3 (es_mesh3d.cu)
 void launch_jacobi3d(bool first, bool last, int grid, cudaStream_t st, const Inst* insts, const int2* work, int nwork,
                      const Scratch* scr, int sweep, int theta_sel);
+// mixed form, 2D: one Jacobi sweep (JF_PER_SWEEP)
+void launch_jacobi_y2d(bool first, bool last, int grid, cudaStream_t st, const Inst* insts, const StagePtrs& single,
+                       const StagePtrs* table, const int2* work, int nwork, const Scratch* scr, int sweep, int theta_sel);
 // FP64 form: one Jacobi sweep
 void launch_jacobi(bool last, int grid, cudaStream_t st, const Inst* insts, const StagePtrs& single,
                    const StagePtrs* table, const int2* work, int nwork, const Scratch* scr, int sweep, int theta_sel);

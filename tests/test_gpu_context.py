@@ -265,3 +265,34 @@ def test_untuned_mesh_tiles_speed(n, mu, nf):
         ctx.es_set_tiles("mesh", *tile)
         all_[tile] = us()
     assert t <= 1.08 * min(all_.values()), (picked, t, all_)
+
+
+@pytest.mark.parametrize("bc", ["periodic", "mixed", "reflect"])
+@pytest.mark.parametrize("mu,nf", [(9, 3), (10, 0), (17, 4), (3, 6)])
+def test_per_sweep_launches_bitwise(bc, mu, nf):
+    """One launch per filter pass and sweep (1 x 1), offered beyond 8 sweeps or 4 filter passes, gives
+    the mesh velocity and Delta t / Delta tau of the fused launches bit for bit; with fewer of both it
+    is refused."""
+    torch = need_gpu()
+    from paper_2202_07989_gb300 import es
+    for n, seed in (((70, 37), 101), ((10, 11), 102), ((200, 199), 103)):
+        pb, JU, J, x, _ = case(2, 2, n, bc, es=True, seed=seed, jump=True)
+        pb = pb.with_(sigma=(W.SIG_RHO1, W.SIG_P), alpha=(60.0, 25.0))
+        ctx = _ctx(pb.with_(mu=mu, nf=nf), 1)
+        G = [to_dev(t, torch) for t in (JU, J, x)]
+        ctx.es_set_mesh_tiles(0)
+        ref = ctx.mesh_redistribute(*G)
+        ctx.es_set_tiles("mesh", 1, 1)
+        assert ctx.es_get_tiles("mesh")[:2] == (1, 1)
+        assert _same(ctx.mesh_redistribute(*G), ref), n
+        with pytest.raises(es.EsError):
+            _ctx(pb.with_(mu=8, nf=4), 1).es_set_tiles("mesh", 1, 1)
+
+
+def test_large_grid_sweeps_run_per_sweep():
+    """On grids where it is the faster by far (2000 x 400 with 16 sweeps: 380 us a mesh step against
+    480), an untuned context runs one launch per sweep; on small ones (64 x 64) the fused launches."""
+    need_gpu()
+    for n, per_sweep in (((2000, 400), True), ((64, 64), False)):
+        ctx = _ctx(W.shock_bubble_2d(*n)[0].with_(mu=16, nf=4), 1)
+        assert (ctx.es_get_tiles("mesh")[:2] == (1, 1)) == per_sweep, n
