@@ -188,8 +188,8 @@ es_status es_get_tuning(const es_ctx* ctx, int* shape, int* S, int* WT, int* gri
 
 /* Fix the flux launch of direction k to tile shape `shape` (0..5) and `grid`
  * CTAs (0 = the library's choice, reported by es_get_tuning: SM count x occupancy
- * of that shape; on a single 3D instance whose lines end in a partial segment the
- * next lower count that shares no factor with the segments per line).
+ * of that shape; on a single 3D instance with more tiles than that, the next lower
+ * count that shares no factor with the segments per line).
  * ES_ERR_ARG when out of range. */
 es_status es_set_tuning(es_ctx* ctx, int k, int shape, int grid);
 

@@ -296,14 +296,15 @@ void prepare_all(int weno)
 int gcd_(int a, int b) { return b == 0 ? a : gcd_(b, a % b); }
 
 // The CTAs of a flux launch along direction k in tiles of S nodes, where the library chooses them:
-// `slots`, or, where a single 3D instance's lines end in a partial segment and there are more tiles
-// than slots, the largest count below that shares no factor with the segments per line.  Tiles are
-// numbered segment by segment, so with a common factor the same CTAs would get every line's partial
-// segment and the others only full ones (direction 1 of 63^3 in the FP64 form, 62 x 4 tiles: 1737 us
-// with 152 CTAs, 1126 us with 151)
+// `slots`, or, where a single 3D instance has more tiles than that, the largest count below that
+// shares no factor with the segments per line.  Tiles are numbered segment by segment, so with a
+// common factor a CTA would get the same segment of every line: the partial one, while others get only
+// full ones (direction 1 of 63^3 in the FP64 form, 62 x 4 tiles: 1737 us with 152 CTAs, 1126 us with 151), or
+// the one where the flow is rough, while others lie in constant states whose interfaces need no WENO
+// values (Riemann 128^3 in the FP64 form, 16 x 15 tiles, no partial segment: 6577 us with 152)
 int auto_grid(const es_ctx* c, int k, int S, long long tiles, int slots)
 {
-    if (c->d != 3 || c->n_inst != 1 || c->hI[0].n[k] % S == 0 || tiles <= slots) return slots;
+    if (c->d != 3 || c->n_inst != 1 || tiles <= slots) return slots;
     const int ns = (c->hI[0].n[k] + S - 1) / S;
     int grid = slots;
     while (grid > 1 && gcd_(grid, ns) != 1) --grid;

@@ -296,3 +296,19 @@ def test_large_grid_sweeps_run_per_sweep():
     for n, per_sweep in (((2000, 400), True), ((64, 64), False)):
         ctx = _ctx(W.shock_bubble_2d(*n)[0].with_(mu=16, nf=4), 1)
         assert (ctx.es_get_tiles("mesh")[:2] == (1, 1)) == per_sweep, n
+
+
+@pytest.mark.parametrize("form", [0, 1])
+def test_library_grid_shares_no_factor_with_segments(form):
+    """Also where every segment is full, so that no CTA stays in one part of the lines: what an
+    interface costs depends on the flow there."""
+    need_gpu()
+    for n in ((128, 128, 128), (112, 60, 56), (208, 40, 40)):
+        ctx = _ctx(W.random_problem(3, 1, n), form)
+        for shape in (None, 0, 4, 5):
+            for k in range(3):
+                if shape is not None:
+                    ctx.es_set_tuning(k, shape)
+                S, WT, grid, _ = ctx.es_get_tiles("flux_k%d" % (k + 1))
+                ns, lines = -(-n[k] // S), -(-n[1 if k == 0 else 0] // WT) * n[1 if k == 2 else 2]
+                assert ns * lines <= grid or math.gcd(grid, ns) == 1, (n, shape, k, S, WT, grid)
