@@ -445,6 +445,13 @@ __device__ __forceinline__ void node_fields(const Inst& I, const R* U, R* nr, in
     if constexpr (!Y::COMPACT) nr[Y::VN * NN + node] = Ar<R>::sq(vn);
 }
 
+// whether a positive product and its reciprocal are well inside the binary64 range (2^-1000 to 2^1000;
+// on the high word, no FP64 comparison)
+__device__ __forceinline__ bool well_inside(double p)
+{
+    return (unsigned int)__double2hiint(p) - (23u << 20) < (2000u << 20);
+}
+
 // pair_flux in the FP64 form, with fewer FP64 instructions: the reciprocals of the two-point sums
 // of every log mean come from one division, and the kinetic terms of E', sum_m ({v_m}^2 -
 // {v_m^2}/2), are half the dot product of the two velocities
@@ -477,11 +484,21 @@ __device__ __forceinline__ void pair_flux64(const Inst& I, const double* nr, int
         const double r = 1.0 / (s0 * sb);
         is = r * s0;
         ir[0] = r * sb;
+        if (!well_inside(s0 * sb)) {
+            is = 1.0 / sb;
+            ir[0] = 1.0 / s0;
+        }
     } else {
         const double s1 = al[1] + ar[1], p = s0 * s1, r = 1.0 / (p * sb), rb = r * sb;
         is = r * p;
         ir[0] = rb * s1;
         ir[1] = rb * s0;
+        // densities whose product leaves the range keep a reciprocal each
+        if (!(well_inside(p) && well_inside(p * sb))) {
+            is = 1.0 / sb;
+            ir[0] = 1.0 / s0;
+            ir[1] = 1.0 / s1;
+        }
     }
     double lr[NS], rt = 0.0, rra = 0.0;
 #pragma unroll

@@ -609,3 +609,21 @@ def test_untuned_3d_tiles_bitwise(form, N, n):
             ctx.es_set_tuning(k, shape)
         got = ctx.es_rhs(*G)
         assert torch.equal(got[0], ref[0]) and torch.equal(got[1], ref[1]), shape
+
+
+@pytest.mark.parametrize("d,N,n", [(2, 1, (20, 17)), (2, 2, (20, 17)), (3, 2, (12, 11, 10))])
+@pytest.mark.parametrize("scale", [2.0 ** -530, 2.0 ** 530])
+def test_ec_residual_scales_with_the_state(d, N, n, scale):
+    """The EC residual is homogeneous in (rho_l, rho v, E): with every density scaled by 2^-530 or
+    2^530 (the product of two densities is then outside the binary64 range) the FP64 residual is
+    the scaled one, to the oracle tolerance (scaling by a power of two is exact but for the rounding
+    of the logarithms of far jumps)."""
+    torch = need_gpu()
+    pb, JU, J, x, xdot = case(d, N, n, "periodic", es=False, seed=111 + N, jump=True)
+    ctx = _ctx(pb, 0)
+    G = [to_dev(t, torch) for t in (JU, J, x, xdot)]
+    ref, refJ = ctx.es_rhs(*G)
+    got, gotJ = ctx.es_rhs(G[0] * scale, *G[1:])
+    assert torch.equal(refJ, gotJ) and ctx.es_poll_status() == 0
+    e = fieldwise((got / scale).cpu().numpy(), ref.cpu().numpy(), N=N, d=d)
+    assert max(e) <= TOL_FP64, e
