@@ -841,7 +841,7 @@ __device__ __forceinline__ void iface_flux(const Inst& I, const R* nb, int NN, i
                     for (int j = 0; j < 6; ++j) {
                         R s_ = R(0);
 #pragma unroll
-                        for (int q = 0; q < NC; ++q) s_ += rc[q] * NR(Y::VV + q, j);
+                        for (int q = 0; q < NC; ++q) s_ = acc_prod(q, rc[q], NR(Y::VV + q, j), s_);
                         wv[j] = s_;
                     }
                     jw = weno_mr_any(wv[5], wv[4], wv[3], wv[2], wv[1], ch1, ch2, ch3, eps) -

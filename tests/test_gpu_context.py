@@ -5,9 +5,10 @@ import time
 
 import pytest
 
+from oracle.oracle import Oracle
 from paper_2202_07989_gb300 import workloads as W
 
-from .helpers import case, need_gpu, to_dev
+from .helpers import TOL_FP64, case, masked_fieldwise, need_gpu, rel_max_err, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -312,3 +313,30 @@ def test_library_grid_shares_no_factor_with_segments(form):
                 S, WT, grid, _ = ctx.es_get_tiles("flux_k%d" % (k + 1))
                 ns, lines = -(-n[k] // S), -(-n[1 if k == 0 else 0] // WT) * n[1 if k == 2 else 2]
                 assert ns * lines <= grid or math.gcd(grid, ns) == 1, (n, shape, k, S, WT, grid)
+
+
+@pytest.mark.parametrize("chi", [(0.009, 0.09, 0.9), (0.5, 0.4, 0.3)])
+@pytest.mark.parametrize("d,N", [(2, 1), (2, 2), (3, 1), (3, 2)])
+def test_weights_that_do_not_sum_to_one(d, N, chi):
+    """FP64 WENO-MR with linear weights that do not sum to one, which then weigh W itself instead of its
+    differences: the oracle's residual in 2D, and the same bits in every tile.  (In 3D such weights
+    make the dissipation depend on the shear directions, which rounding picks where the normal is x_3.)"""
+    torch = need_gpu()
+    n = (41, 29) if d == 2 else (40, 11, 10)
+    pb, JU, J, x, xdot = case(d, N, n, "mixed", es=True, seed=121 + N, jump=True)
+    pb = pb.with_(chi=chi)
+    ctx = _ctx(pb, 0)
+    G = [to_dev(t, torch) for t in (JU, J, x, xdot)]
+    ref = ctx.es_rhs(*G)
+    if d == 2:
+        want, wantJ, mg = Oracle(pb).rhs_margins(JU, J, x, xdot)
+        e, skipped = masked_fieldwise(ref[0].cpu().numpy(), want, mg, N, d)
+        assert max(e + [rel_max_err(ref[1].cpu().numpy(), wantJ)]) <= TOL_FP64 and skipped <= 0.01 * pb.ncell, (e, skipped)
+    if d == 2:
+        tiles = [[("stage", t)] for t in ((0, 0),) + STAGE_TILES + STAGE_TILES_FP64]
+    else:
+        tiles = [[("flux_k%d" % (k + 1), t) for k in range(3)] for t in ((62, 4), (30, 8), (15, 16), (255, 1), (7, 13))]
+    for t in tiles:
+        for launch, extent in t:
+            ctx.es_set_tiles(launch, *extent)
+        assert _same(ctx.es_rhs(*G), ref), t
