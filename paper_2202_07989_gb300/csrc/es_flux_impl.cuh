@@ -101,8 +101,9 @@ __device__ __forceinline__ void flux_stage(const FluxLaunch& L, int k, int wi, d
     cp_async_commit();
 }
 
-// t / n for 0 <= t < 4096 and 1 <= n <= 512, given r = 1/n in binary32: (t + 1/2) r is off the exact
-// quotient by less than 4096 * 2^-23 < 1 / (2n), so its integer part is t / n
+// t / n for 0 <= t < 2^21 and any n >= 1, given r = 1/n in binary32: (t + 1/2) r, with two roundings of
+// 2^-24, is off (t + 1/2) / n by less than 1 / (4n), and that lies at least 1 / (2n) from an integer,
+// so its integer part is t / n.  (The FP64 3D tiles divide by up to 3 * 255 + 6 = 771.)
 __device__ __forceinline__ int div_small(int t, float r) { return (int)(((float)t + 0.5f) * r); }
 
 // Phases of one tile: (1) node states, entropy variables and metrics into shared memory;
@@ -120,7 +121,7 @@ __global__ void __launch_bounds__(FLUX_TPB, (sizeof(R) == 4 ? (D == 3 ? 4 : 3) :
     using TL = Tile<S_, WT_>;
     constexpr int NC = Y::NC, NN = TL::NN, NI = TL::NI, NF = Y::NF, NP = TL::NP;
     constexpr bool PRIM = D == 3 && std::is_same<R, float>::value;
-    static_assert(NP < 4096 && 3 * S_ + 6 <= 512, "div_small");
+    static_assert(NP < (1 << 21) && NN < (1 << 21), "div_small");
     const int S = S_ > 0 ? S_ : L.S, WT = S_ > 0 ? WT_ : L.WT, NPL = 3 * S + 6;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double* gt = reinterpret_cast<double*>(smem_raw);           // [NI] GCL flux of J xi_k/t
