@@ -627,3 +627,48 @@ def test_ec_residual_scales_with_the_state(d, N, n, scale):
     assert torch.equal(refJ, gotJ) and ctx.es_poll_status() == 0
     e = fieldwise((got / scale).cpu().numpy(), ref.cpu().numpy(), N=N, d=d)
     assert max(e) <= TOL_FP64, e
+
+
+@pytest.mark.parametrize("d,N", [(2, 1), (2, 2), (3, 2)])
+def test_log_mean_thresholds(d, N):
+    """FP64 log means at the edges of their branches: densities and pressures whose jumps
+    |a - b| / (a + b) lie at 2^-7 and 2^-3 (four- and nine-term series, logarithms), one rounding to
+    either side, against the oracle's EC residual."""
+    torch = need_gpu()
+    pb, JU, J, x, xdot = case(d, N, GRIDS[d], "periodic", es=False, seed=131 + N)
+    rng = np.random.default_rng(5)
+    f = np.concatenate([2.0 ** -q * (1 + np.arange(-2, 3) * 2.0 ** -52) for q in (3, 7)] + [[0.0]])
+    U = JU / J
+    U[:] = U.mean(axis=(1, 2, 3), keepdims=True)
+    ratio = (1 + f) / (1 - f)
+    pick = lambda: ratio[rng.integers(0, f.size, size=J.shape[-3:])]
+    for l in range(pb.N):
+        U[l] *= pick()
+    U[pb.N:pb.N + d] = 0.0
+    U[pb.N + d] *= pick()
+    want, wantJ = Oracle(pb).rhs(U * J, J, x, xdot)
+    ctx = _ctx(pb)
+    got, gotJ = ctx.es_rhs(to_dev(U * J, torch), to_dev(J, torch), to_dev(x, torch), to_dev(xdot, torch))
+    e = fieldwise(got.cpu().numpy(), want, N=pb.N, d=d) + [rel_max_err(gotJ.cpu().numpy(), wantJ)]
+    assert max(e) <= TOL_FP64, e
+
+
+@pytest.mark.parametrize("d,N", [(2, 1), (2, 2), (3, 2)])
+@pytest.mark.parametrize("v", [2.0 ** -83, 2.0 ** 83])
+def test_weno_denominators_out_of_range(d, N, v):
+    """FP64 WENO-MR where the product of the two values' denominators (degree 12 to 16 in the jumps)
+    leaves the binary64 range and each takes its own division, against the oracle: a change of the
+    unit of time scales velocities by v, energies, c_v and epsilon by v^2 and the scaled entropy
+    variables by v, and leaves beta and the logarithms as they are."""
+    torch = need_gpu()
+    pb, JU, J, x, xdot = case(d, N, GRIDS[d], "periodic", es=True, seed=141 + N, jump=True)
+    pb = pb.with_(cv=tuple(c * v * v for c in pb.cv), weno_eps=pb.weno_eps * v * v)
+    JU = JU.copy()
+    JU[N:N + d] *= v
+    JU[N + d] *= v * v
+    want, wantJ, mg = Oracle(pb).rhs_margins(JU, J, x, xdot * v)
+    ctx = _ctx(pb)
+    got, gotJ = ctx.es_rhs(to_dev(JU, torch), to_dev(J, torch), to_dev(x, torch), to_dev(xdot * v, torch))
+    e, skipped = masked_fieldwise(got.cpu().numpy(), want, mg, pb.N, pb.d)
+    assert max(e + [rel_max_err(gotJ.cpu().numpy(), wantJ)]) <= TOL_FP64, e
+    assert skipped <= 0.01 * pb.ncell, skipped
