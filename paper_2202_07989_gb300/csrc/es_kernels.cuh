@@ -24,7 +24,8 @@ constexpr int SHAPE_DEFAULT_KN = 3;    // directions 2, 3: 30 nodes x 8 neighbou
 // CTAs in each shape relative to 16 x 12 tiles, binary32 and binary64, measured on grids of one wave
 // (single-species FP64 launches, us: 16 x 12 139.6, 8 x 8 64, 12 x 8 82, 16 x 8 110, 16 x 14 158,
 // 24 x 15 237; mixed residuals, metrics pass included, 21.9, 15.6, 16.3, 19.5), by which a context that nobody tuned
-// picks its tiles: the least waves x cost (pick_fused in es_api.cu).
+// picks its tiles: the least waves x cost (pick_fused in es_api.cu).  Two-species and WENO-JS residuals
+// take the same picks: on 21 grids (32^2 .. 1200 x 480) none was more than 1% slower than 16 x 12.
 constexpr int NFSHAPE = 5;
 // The last two are for the FP64 form only, whose phases cost whole warps on each of the SM's four
 // FP64 pipes: 16 x 14 tiles need no more rounds than 16 x 12 for 17% more nodes (two of interfaces a

@@ -978,9 +978,9 @@ __device__ __forceinline__ bool grid_edge(int g0, int n0, bool per0, int g1, int
 // A mesh step of more than 8 sweeps runs in several launches of about equal sweep counts
 // (jacobi_fused2d): every launch but the last stores y, the first also the filtered Theta, and
 // every launch but the first starts from the stored y (src) and Theta (F < 0).  The last one
-// forms the limiter bounds of Sec. 4.  One launch per filter pass and sweep, as such steps ran
-// before, is bound by launch latency: the 64^2 vortex step with ten
-// sweeps and three filter passes went from 141.2 us (14 such launches) to 108.9 us (2 launches).
+// forms the limiter bounds of Sec. 4.  On small grids one launch per filter pass and sweep is bound by
+// launch latency (64^2 mesh step of ten sweeps and three passes: 84 us in 14 such launches, 43 in 2
+// fused ones); large ones take it (JF_PER_SWEEP).
 template <int TX, int TY, int TPB>
 __global__ void __launch_bounds__(TPB, 1024 / TPB) jacobi_fused2d_kernel(const Inst* __restrict__ insts, StagePtrs single,
                                                                           const StagePtrs* __restrict__ table,
